@@ -611,11 +611,16 @@ __device__ __forceinline__ void cache_unpin(const Dev &d, uint32_t line) {
   atomicAdd(&d.tag[line], (unsigned long long)(-(int64_t)PIN1));
 }
 
-// Put back a victim we claimed but could not use (keeps transient pin bits of others).
+// Give up a victim we claimed but could not use (keeps transient pin bits of others).  A
+// MODIFIED victim gets its tag back: its page's in-flight entry, held by the caller, has
+// kept everyone from reading the page meanwhile.  A clean one has no such entry: another
+// thread may have missed on its page and be filling a second way with it, and two valid
+// copies lose updates.  Its way is left INVALID.
 __device__ __forceinline__ void cache_unclaim(const Dev &d, uint32_t line, uint64_t old_tag) {
   uint64_t cur = ld_rlx64(&d.tag[line]);
+  const uint64_t back = tag_state(old_tag) == ST_MODIFIED ? old_tag & ~PIN_MASK : 0;
   for (int i = 0; i < 64; ++i) {
-    uint64_t want = (old_tag & ~PIN_MASK) | (cur & PIN_MASK);
+    uint64_t want = back | (cur & PIN_MASK);
     uint64_t got = atomicCAS(&d.tag[line], (unsigned long long)cur, (unsigned long long)want);
     if (got == cur) return;
     cur = got;
