@@ -116,8 +116,8 @@ typedef struct {
   uint32_t share_slots;     /* Share Table entries for user buffers (Sec. 3.4.1); 0 = no
                                Share Table (it is an option, as in the paper)        */
   uint32_t emu_extra_engines; /* application warps a call leaves idle that also serve the
-                               emulated device, at most: 0 = one per CTA of the launch,
-                               AGILE_NO_EXTRA_ENGINES = none (only warp 0 of each CTA) */
+                               emulated device, at most: 0 or AGILE_NO_EXTRA_ENGINES =
+                               none (the launch's service CTAs are its engines)        */
   uint32_t prefetch_queues; /* queue pairs that carry requests made ahead of need (the
                                asynchronous lookahead of the drivers, agile_prefetch);
                                the device serves the other, demand queues first (NVMe

@@ -111,17 +111,21 @@ int launch_user(agile_ctx *ctx, const App &app, void *stream, uint32_t app_warps
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return AGILE_ECUDA;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return AGILE_ECUDA;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, engine_kernel<App>, kThreads, 0) != cudaSuccess ||
+  if (engine_shared<App>() > 0 &&
+      cudaFuncSetAttribute(engine_kernel<App>, cudaFuncAttributeMaxDynamicSharedMemorySize, engine_shared<App>()) !=
+          cudaSuccess)
+    return AGILE_ECUDA;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, engine_kernel<App>, EngineShape<App>::threads,
+                                                    engine_shared<App>()) != cudaSuccess ||
       per_sm <= 0)
     return AGILE_ECUDA;
   d.app_active = app_warps;
-  if (d.extra_engines == 0xFFFFFFFFu) d.extra_engines = (uint32_t)(per_sm * sms);  // default: one per CTA
   r = agile_run_reset(ctx, stream);
   if (r) return r;
   App a = app;
   void *args[] = {(void *)&d, (void *)&a};
-  if (cudaLaunchCooperativeKernel((const void *)engine_kernel<App>, dim3(per_sm * sms), dim3(kThreads), args, 0,
-                                  (cudaStream_t)stream) != cudaSuccess)
+  if (cudaLaunchCooperativeKernel((const void *)engine_kernel<App>, dim3(per_sm * sms),
+                                  dim3(EngineShape<App>::threads), args, engine_shared<App>(), (cudaStream_t)stream) != cudaSuccess)
     return AGILE_ECUDA;
   return AGILE_OK;
 }

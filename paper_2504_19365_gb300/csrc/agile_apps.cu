@@ -30,7 +30,7 @@ struct EmbApp {
   // no request ahead of need: the launch uses every queue pair for demand
   bool demand_only() const { return mode == AGILE_SYNC; }
   uint32_t ahead;  // rows requested ahead of the one being summed (ASYNC), 1..32
-  uint32_t group;  // rows pinned together at most (cache-sized), 1..32
+  uint32_t group;  // pages requested and not yet used, at most (cache-sized), 1..32
   // bags left by the resident pass: positions 0 .. *list_n - 1 name bags list[pos]
   // (nullptr: every bag, position = bag); n_bags bounds the positions
   const uint32_t *list = nullptr;
@@ -74,7 +74,7 @@ struct EmbApp {
           want = false;
         }
         uint32_t outcome = 0;
-        if (!warp_request(d, want, row_page(r), a.q0, false, a.deadline, nullptr, nullptr, &outcome, true, true))
+        if (!warp_request(d, want, row_page(r), a.q0, false, a.deadline, nullptr, nullptr, &outcome, true, true, group))
           return false;
         bo.result(outcome);
       }
@@ -160,15 +160,12 @@ struct EmbApp {
       }
       uint32_t cnt = (uint32_t)min((int64_t)32, e - i0);
       uint64_t byte = r * dim * 4;
-      for (uint32_t g0 = 0; g0 < cnt; g0 += group) {
-        uint32_t g1 = min(cnt, g0 + group);
-        // keep the pages of the next `ahead` rows of the stream requested
-        if (async && !issue_rows(d, a, pf, g1 - g0, bo)) return false;
-        bool missed = false;
-        if (!gather_sum<MF4>(d, a, g0, g1, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, &missed))
-          return false;
-        if (missed) bo.missed();
-      }
+      // keep the pages of the next `ahead` rows of the stream requested
+      if (async && !issue_rows(d, a, pf, cnt, bo)) return false;
+      bool missed = false;
+      if (!gather_sum<MF4>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, group, &missed))
+        return false;
+      if (missed) bo.missed();
     }
     store_out(b, acc, nf4);
     return true;
@@ -276,7 +273,7 @@ struct PipeApp {
   uint32_t mode;
   // no request ahead of need: the launch uses every queue pair for demand
   bool demand_only() const { return mode == AGILE_SYNC; }
-  uint32_t group;     // rows pinned together at most (cache-sized), 1..32
+  uint32_t group;     // pages requested and not yet used, at most (cache-sized), 1..32
   uint32_t ahead;     // async: rows of the warp's row stream requested ahead (cache-sized)
 
   __device__ __forceinline__ uint64_t row_page(uint32_t k, uint64_t r) const {
@@ -307,7 +304,7 @@ struct PipeApp {
           want = false;
         }
         uint32_t outcome = 0;
-        if (!warp_request(d, want, row_page(k, r), a.q0, false, a.deadline, nullptr, nullptr, &outcome, true, true))
+        if (!warp_request(d, want, row_page(k, r), a.q0, false, a.deadline, nullptr, nullptr, &outcome, true, true, group))
           return false;
         bo.result(outcome);
       }
@@ -347,14 +344,11 @@ struct PipeApp {
             r = 0;
           }
           uint64_t byte = (uint64_t)k * tstride + r * dim * 4;
-          for (uint32_t g0 = 0; g0 < cnt; g0 += group) {
-            uint32_t g1 = min(cnt, g0 + group);
-            if (async && !issue_ahead(d, a, pf, g1 - g0, units, bo)) return;
-            bool missed = false;
-            if (!gather_sum<MF4>(d, a, g0, g1, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, &missed))
-              return;
-            if (missed) bo.missed();
-          }
+          if (async && !issue_ahead(d, a, pf, cnt, units, bo)) return;
+          bool missed = false;
+          if (!gather_sum<MF4>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, group, &missed))
+            return;
+          if (missed) bo.missed();
         }
         // compute phase on this table's pooled row
 #pragma unroll
@@ -511,7 +505,7 @@ struct BfsAppT {
       uint64_t p = __shfl_sync(kFull, nxt, __ffs(m) - 1);
       release(d, pc);
       uint32_t line;
-      if (!warp_pin_page<true>(d, p, a.q0, a.deadline, line)) return false;
+      if (!warp_pin_page(d, p, a.q0, a.deadline, line)) return false;
       pc.page = p;
       pc.line = line;
       pc.valid = true;
@@ -898,6 +892,7 @@ struct SpmvAppT {
   static constexpr uint32_t kChunk = 128;
   static constexpr uint32_t kHub = 1024;
   static constexpr uint32_t kSlice = 1024;  // = the products buffer of a warp
+  static constexpr int kSharedPerWarp = kSlice * 4;
 
   struct Pin {
     uint64_t page;
@@ -969,7 +964,7 @@ struct SpmvAppT {
       if (warp_probe_pin(d, p, line) != P_HIT) {
         release(d, o1);
         release(d, o2);
-        if (!warp_pin_page<true>(d, p, a.q0, a.deadline, line)) return false;
+        if (!warp_pin_page(d, p, a.q0, a.deadline, line)) return false;
       }
       pc.page = p;
       pc.line = line;
@@ -1152,8 +1147,8 @@ struct SpmvAppT {
 
   // take queued slices until every slice is taken (the BFS slice queue, one level)
   __device__ bool help_hubs(const Dev &d, const AppCtx &a, Pin &po, Pin &pcol, Pin &pval) const {
-    __shared__ float prod_buf[kWarps][kSlice];  // products of the slice a warp holds
-    float *buf = prod_buf[threadIdx.x >> 5];
+    extern __shared__ float prod_buf[];  // products of the slice a warp holds
+    float *buf = prod_buf + (threadIdx.x >> 5) * kSlice;
     unsigned l = lane_id();
     const uint64_t ep = launch_epoch(d);
     const uint64_t want_tag = (ep << 32) | 1u;
@@ -1517,8 +1512,8 @@ __global__ void bfs_init_kernel(int32_t *level, uint32_t *vis, uint32_t n, int32
   if (i < (n + 31ull) / 32) vis[i] = (i == (uint64_t)src / 32) ? 1u << (src % 32) : 0u;
 }
 
-// rows a warp pins together: with `warps` warps each holding that many lines at once,
-// at most half of the cache is pinned
+// pages a warp requests before it uses them: with `warps` warps each holding that many
+// lines at once, at most half of the cache is waited for
 uint32_t pin_group(const agile_ctx *c, uint32_t warps) {
   uint64_t g = c->dev.nlines / (2ull * std::max<uint32_t>(1, warps));
   return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(32, g));
@@ -1690,7 +1685,7 @@ int agile_embedding_bag(agile_ctx *c, uint64_t table_byte0, uint32_t rows, uint3
     // three CTAs per SM (fewer registers a thread, so slower service warps) pay off only
     // when the cache holds enough lines for more warps than two CTAs per SM give
     uint64_t want = c->cfg.app_warps ? c->cfg.app_warps : warps;
-    if (want > (uint64_t)std::max(0, engine_grid<EmbApp<1, 2>>(c)) * (kWarps - 1)) return go(EmbApp<1, 3>{});
+    if (want > app_warps_of_grid<EmbApp<1, 2>>(c)) return go(EmbApp<1, 3>{});
     return go(EmbApp<1, 2>{});
   }
   if (dim <= 256) return go(EmbApp<2>{});

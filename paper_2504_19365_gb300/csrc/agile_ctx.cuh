@@ -59,7 +59,12 @@ int engine_grid(agile_ctx *c) {
   static int per_sm = -1;  // one value per instantiation
   if (per_sm < 0) {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, engine_kernel<App>, kThreads, 0) != cudaSuccess)
+    if (engine_shared<App>() > 0 &&
+        cudaFuncSetAttribute(engine_kernel<App>, cudaFuncAttributeMaxDynamicSharedMemorySize, engine_shared<App>()) !=
+            cudaSuccess)
+      return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, engine_kernel<App>, EngineShape<App>::threads,
+                                                      engine_shared<App>()) != cudaSuccess)
       return 0;
     per_sm = n;
   }
@@ -71,8 +76,13 @@ int engine_grid(agile_ctx *c) {
 // Application warps a launch of this instantiation runs when the call wants `active`
 // (0 = all): the context's app_warps setting overrides `active`, the grid bounds both.
 template <class App>
+uint64_t app_warps_of_grid(agile_ctx *c) {
+  const Roles r = engine_roles((uint32_t)std::max(0, engine_grid<App>(c)), EngineShape<App>::warps);
+  return (uint64_t)r.app_ctas * r.per_cta;
+}
+template <class App>
 uint32_t running_app_warps(agile_ctx *c, uint32_t active) {
-  uint64_t n_app = (uint64_t)std::max(0, engine_grid<App>(c)) * (kWarps - 1);
+  uint64_t n_app = app_warps_of_grid<App>(c);
   uint64_t want = c->cfg.app_warps ? c->cfg.app_warps : active;
   return (uint32_t)std::max<uint64_t>(1, want && want < n_app ? want : n_app);
 }
@@ -111,14 +121,13 @@ int launch_engine(agile_ctx *c, const App &app, void *stream, uint32_t active = 
   AGILE_CUDA_TRY(cudaGetLastError());
   Dev d = c->dev;
   d.app_active = c->cfg.app_warps ? c->cfg.app_warps : active;
-  if (d.extra_engines == 0xFFFFFFFFu) d.extra_engines = (uint32_t)grid;  // default: one per CTA
   if constexpr (has_demand_only<App>::value) {
     if (app.demand_only()) d.Qp = 0;
   }
   App a = app;
   void *args[] = {(void *)&d, (void *)&a};
-  AGILE_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)engine_kernel<App>, dim3(grid), dim3(kThreads),
-                                             args, 0, s));
+  AGILE_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)engine_kernel<App>, dim3(grid),
+                                             dim3(EngineShape<App>::threads), args, engine_shared<App>(), s));
   return AGILE_OK;
 }
 

@@ -4,17 +4,18 @@
 //   lines      [nlines * 4096]      cache data, one 4 KiB line per store page (Sec. 2.3.3)
 //   tag        [nlines] u64         {page:44 | pin:16 | wb:1 | ref:1 | state:2} (Sec. 3.4)
 //   hand       [sets]   u32         clock hand per set (Sec. 4.4, clock policy)
-//   sh_key/val [buckets*4] u64      in-flight share table, 4 slots per bucket (Sec. 3.4.1)
+//   sh_key     [buckets] u64        in-flight share table, 4 slots of 16 bits per bucket
+//   sh_val     [buckets*4] u64      (Sec. 3.4.1), and the token of each slot's read
 //   sq         [Q * depth] 64 B     NVMe submission entries (Sec. 2.1)
 //   cq         [Q * 2*depth] 16 B   NVMe completion entries with phase bit (Sec. 2.1)
-//   sqe_state  [Q * depth] u64      {ticket:62 | EMPTY/UPDATED/ISSUED} (Sec. 3.3.1)
+//   sqe_state  [Q * depth] u64      {ticket:62 | EMPTY/UPDATED/WRITTEN} (Sec. 3.3.1)
 //   cmd_ctx    [Q * depth] u64      what a completion releases (line fill, write-back)
 //   cmpl       [Q * depth] u64      completion word = transaction barrier (Sec. 3.2.1)
 //   sq_resv    [Q] u64              {in flight:32 | next ticket:32}
-//   sq_tail/sq_lock/sq_db [Q] u32   doorbell-lock holder's tail, the lock, doorbell
+//   sq_db      [Q] u32              doorbell: commands issued so far (slot = count mod depth)
 //   cq_db      [Q] u32              CQ head doorbell
 //   cq_poll    [Q*4] u32            Alg. 1 state {offset, mask, phase}
-//   emu*                            emulated device: fetch/seen/CQ-slot counters, timing
+//   emu_*      [Q] u32              emulated device: fetch/seen/CQ-slot counters, timing
 //   staging    [Q * depth * 4096]   write-back sources, one page per submission slot
 #pragma once
 #include <cstdint>
@@ -23,8 +24,9 @@
 namespace agile {
 
 constexpr uint32_t kPage = 4096;
-constexpr int kWarps = 8;             // warps per CTA: warp 0 = service, 1..7 = app
-constexpr int kThreads = kWarps * 32;
+// An engine CTA fills its SM: kWarps warps times the occupancy its application is compiled
+// for (MinBlocks, 2 by default: 16 warps of 128 registers).
+constexpr int kWarps = 8;
 constexpr unsigned kFull = 0xffffffffu;
 
 // ---------------------------------------------------------------- tag word (Sec. 3.4)
@@ -45,7 +47,7 @@ __host__ __device__ __forceinline__ uint64_t tag_make(uint64_t page, uint64_t st
 constexpr uint32_t kPolicyClock = 0, kPolicyFifo = 1;
 
 // ---------------------------------------------------------------- queues (Sec. 3.3.1)
-constexpr uint64_t SQE_EMPTY = 0, SQE_UPDATED = 1, SQE_ISSUED = 2;
+constexpr uint64_t SQE_EMPTY = 0, SQE_UPDATED = 1, SQE_WRITTEN = 2;
 constexpr uint32_t OP_FLUSH = 0x00, OP_WRITE = 0x01, OP_READ = 0x02;
 
 // command context: what the completion of a command releases (CTX_BUF: a read into a
@@ -67,9 +69,9 @@ enum Stat {
 
 // per-launch state, zeroed before every launch (and numbered) by run_reset_kernel
 struct RunState {
-  uint32_t app_done;      // app warps finished
+  uint32_t app_done;      // CTAs whose application warps have all finished
   uint32_t error;         // first error code (negated AGILE_E*), 0 = none
-  uint32_t bar_count;     // grid barrier arrivals
+  uint32_t bar_count;     // grid barrier arrivals (CTAs)
   uint32_t bar_gen;       // grid barrier generation
   uint32_t work[4];       // dynamic work counters
   unsigned long long acc[4];  // accumulators (edges scanned, discovered vertices, ...)
@@ -105,7 +107,8 @@ struct Dev {
   uint32_t sets, ways;
   unsigned long long *sh_key;
   unsigned long long *sh_val;
-  uint32_t sh_mask;  // buckets - 1 (power of two)
+  uint32_t sh_bits;  // log2 of buckets * 2^15: the page numbers the table tells apart
+  uint64_t sh_mul;   // odd: page * sh_mul mod 2^sh_bits = {bucket, 15-bit key}
   // queues
   uint32_t Q, depth, dmask, dlog;
   uint32_t Qp;       // queues [Q - Qp, Q) carry prefetches, served after the demand queues
@@ -116,8 +119,10 @@ struct Dev {
   unsigned long long *cmd_ctx;
   unsigned long long *cmpl;
   unsigned long long *sq_resv;
-  uint32_t *sq_tail, *sq_lock, *sq_db, *cq_db, *cq_poll;
-  uint32_t *emu;  // [Q*4] device counters {fetch, seen, cq slot, -}
+  uint32_t *sq_db, *cq_db, *cq_poll;
+  // device counters per queue, unwrapped: next command to fetch, doorbell seen, next CQ
+  // slot (arrays of their own: engines scan the first one next to the doorbells)
+  uint32_t *emu_fetch, *emu_seen, *emu_cqt;
   unsigned long long *emu_busy;     // [Q] ns at which the queue's device pipe is free
   unsigned long long *emu_arrival;  // [Q*depth] ns at which the device saw the command
   uint8_t *staging;
@@ -158,6 +163,24 @@ struct Dev {
   uint32_t extra_engines;  // idle application warps that may also serve the device
   uint64_t session_ns;  // length of a long-running launch (serving loop); 0 = timeout_ns
 };
+
+// What an engine CTA keeps in shared memory.
+// dev: the launch's Dev, for the functions that are kept out of line.  They cannot read
+// the kernel's parameter bank, and through a pointer to it every field would be a load
+// that each fence sends back to L2 (issuing a command took 5.5 us that way, most of it
+// such reloads).
+struct CtaState {
+  Dev dev;
+  uint32_t done;                     // application warps of this CTA that have finished
+  uint32_t bar_count, bar_gen;       // grid barrier: arrivals in this CTA, generation
+  uint32_t active;                   // application warps of this CTA that take part
+  uint32_t ctas_active;              // CTAs with such warps
+};
+__device__ __forceinline__ CtaState &cta_state() {
+  __shared__ CtaState cs;
+  return cs;
+}
+__device__ __forceinline__ const Dev &shared_dev() { return cta_state().dev; }
 
 // ---------------------------------------------------------------- PTX helpers
 __device__ __forceinline__ uint64_t gtimer() {
@@ -200,6 +223,11 @@ __device__ __forceinline__ void st_rlx32(uint32_t *p, uint32_t v) {
 __device__ __forceinline__ uint64_t atom_add_acq(unsigned long long *p, uint64_t v) {
   uint64_t old;
   asm volatile("atom.acquire.gpu.global.add.u64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
+  return old;
+}
+__device__ __forceinline__ uint64_t atom_cas_acq(unsigned long long *p, uint64_t cmp, uint64_t v) {
+  uint64_t old;
+  asm volatile("atom.acquire.gpu.global.cas.b64 %0, [%1], %2, %3;" : "=l"(old) : "l"(p), "l"(cmp), "l"(v) : "memory");
   return old;
 }
 __device__ __forceinline__ void fence_sc() { asm volatile("fence.sc.gpu;" ::: "memory"); }
@@ -321,10 +349,10 @@ __device__ __forceinline__ void lane_copy_page(void *dst, const void *src) {
 // Alg. 2, check_full: reserve n consecutive slots of queue q.  A slot is free when
 // the command that used it last has completed (state EMPTY) and fewer than depth-1
 // commands are outstanding (the NVMe full rule).  Never waits.
-__device__ __forceinline__ bool sq_try_reserve(const Dev &d, uint32_t q, uint32_t n,
+// `w`: the queue's reservation word as read before.
+__device__ __forceinline__ bool sq_try_reserve(const Dev &d, uint32_t q, uint32_t n, uint64_t w,
                                                uint32_t &slot, uint32_t &ticket) {
   unsigned long long *rp = &d.sq_resv[q];
-  uint64_t w = ld_rlx64(rp);
   for (int tries = 0; tries < 4; ++tries) {
     uint32_t t = (uint32_t)w, infl = (uint32_t)(w >> 32);
     if (infl + n > d.depth - 1) return false;
@@ -358,21 +386,38 @@ __host__ __device__ __forceinline__ uint64_t block_of_page(const Dev &d, uint64_
 // only use device time that demand leaves idle) -- start at the one nearest the
 // thread's own queue, on a full queue try the class's next one of the device; false
 // after one pass over them.
-__device__ __forceinline__ bool sq_reserve_dev(const Dev &d, uint32_t q0, uint32_t dv, uint32_t n, uint32_t &q,
-                                               uint32_t &slot, uint32_t &ticket, bool pf = false) {
-  const uint32_t nd = d.ndev > 1 ? d.ndev : 1u;
-  const uint32_t base = pf && d.Qp ? d.Q - d.Qp : 0u;
+struct SqPick {
+  uint32_t base, per, nd, k0;  // queue of the class's k-th of the device: base + k * nd + dv
+};
+__device__ __forceinline__ SqPick sq_pick(const Dev &d, uint32_t q0, bool pf) {
+  SqPick p;
+  p.nd = d.ndev > 1 ? d.ndev : 1u;
+  p.base = pf && d.Qp ? d.Q - d.Qp : 0u;
   const uint32_t cnt = d.Qp ? (pf ? d.Qp : d.Q - d.Qp) : d.Q;
-  const uint32_t per = cnt / nd;  // queues of one device in the class
-  uint32_t k0 = (q0 / nd) % per;
+  if (p.nd == 1) {
+    p.per = cnt;
+    p.k0 = q0 < cnt ? q0 : q0 % cnt;
+  } else {
+    p.per = cnt / p.nd;  // queues of one device in the class
+    p.k0 = (q0 / p.nd) % p.per;
+  }
+  return p;
+}
+// `w0`: the reservation word of the first queue, if the caller has read it (its load then
+// overlaps the caller's other loads), else kNoWord
+constexpr uint64_t kNoWord = ~0ull;
+__device__ __forceinline__ bool sq_reserve_dev(const Dev &d, uint32_t q0, uint32_t dv, uint32_t n, uint32_t &q,
+                                               uint32_t &slot, uint32_t &ticket, bool pf = false,
+                                               uint64_t w0 = kNoWord) {
+  const SqPick p = sq_pick(d, q0, pf);
   // a request made ahead of need tries two queues: when they are full the device is
   // saturated and the request is dropped (a hint), not spread over every queue
-  const uint32_t tries = pf ? min(per, 2u) : per;
+  const uint32_t tries = pf ? min(p.per, 2u) : p.per;
   for (uint32_t k = 0; k < tries; ++k) {
-    uint32_t kk = k0 + k;
-    if (kk >= per) kk -= per;
-    uint32_t qq = base + kk * nd + dv;
-    if (sq_try_reserve(d, qq, n, slot, ticket)) {
+    uint32_t kk = p.k0 + k;
+    if (kk >= p.per) kk -= p.per;
+    uint32_t qq = p.base + kk * p.nd + dv;
+    if (sq_try_reserve(d, qq, n, k == 0 && w0 != kNoWord ? w0 : ld_rlx64(&d.sq_resv[qq]), slot, ticket)) {
       q = qq;
       return true;
     }
@@ -380,24 +425,23 @@ __device__ __forceinline__ bool sq_reserve_dev(const Dev &d, uint32_t q0, uint32
   atomicAdd(stat_ptr(d, S_SQ_FULL), 1ull);
   return false;
 }
+__device__ __forceinline__ uint64_t sq_first_word(const Dev &d, uint32_t q0, uint32_t dv, bool pf) {
+  const SqPick p = sq_pick(d, q0, pf);
+  return ld_rlx64(&d.sq_resv[p.base + p.k0 * p.nd + dv]);
+}
 
 // The first queue sq_reserve_dev tries for a request of this class holds more than
 // 3/4 of its depth in flight: a request made ahead of need is then dropped before it
 // claims a line (one load instead of a claim, a failed reservation and an unclaim).
 __device__ __forceinline__ bool sq_crowded(const Dev &d, uint32_t q0, uint32_t dv, bool pf) {
-  const uint32_t nd = d.ndev > 1 ? d.ndev : 1u;
-  const uint32_t base = pf && d.Qp ? d.Q - d.Qp : 0u;
-  const uint32_t cnt = d.Qp ? (pf ? d.Qp : d.Q - d.Qp) : d.Q;
-  const uint32_t per = cnt / nd;
-  const uint32_t qq = base + ((q0 / nd) % per) * nd + dv;
-  return (uint32_t)(ld_rlx64(&d.sq_resv[qq]) >> 32) > (d.depth - 1) / 4 * 3;
+  return (uint32_t)(sq_first_word(d, q0, dv, pf) >> 32) > (d.depth - 1) / 4 * 3;
 }
 
-// Alg. 2, enqueue_cmd + update_SQE: write the 64-byte command, then publish the slot
-// as UPDATED.  CID = slot index (unique while the command is outstanding).
-__device__ __forceinline__ void sq_commit(const Dev &d, uint32_t q, uint32_t slot, uint32_t ticket,
-                                          uint32_t opcode, uint64_t prp1, uint64_t page,
-                                          uint64_t ctx) {
+// Alg. 2, enqueue_cmd: write the 64-byte command into its reserved slot.  CID = slot index
+// (unique while the command is outstanding).  sq_ring, by the same thread, issues it.
+__device__ __forceinline__ void sq_write(const Dev &d, uint32_t q, uint32_t slot, uint32_t ticket,
+                                         uint32_t opcode, uint64_t prp1, uint64_t page,
+                                         uint64_t ctx) {
   uint64_t i = (uint64_t)q * d.depth + slot;
   uint32_t *e = d.sq[i].dw;
   uint64_t slba = block_of_page(d, page) * (kPage / 512);
@@ -412,126 +456,107 @@ __device__ __forceinline__ void sq_commit(const Dev &d, uint32_t q, uint32_t slo
   st_cg16(e + 8, c);
   st_cg16(e + 12, f);
   st_rlx64(&d.cmd_ctx[i], ctx);
-  // the release orders the command's stores (and the caller's earlier ones) before the
-  // state: whoever acquires UPDATED -- the doorbell-lock holder, then the device through
-  // the doorbell -- sees them
-  st_rel64(&d.sqe_state[i], ((uint64_t)ticket << 2) | SQE_UPDATED);
+  st_rlx64(&d.sqe_state[i], ((uint64_t)ticket << 2) | SQE_WRITTEN);
 }
 
-// Alg. 2, move_SQ_tail: the doorbell-lock holder turns UPDATED slots into ISSUED from
-// the tail up to the first slot that is not UPDATED, then writes the doorbell once.
-__device__ __forceinline__ void sq_move_tail(const Dev &d, uint32_t q) {
-  uint32_t t = ld_rlx32(&d.sq_tail[q]);
-  uint32_t n = 0;
-  while (n < d.depth) {
-    uint64_t i = (uint64_t)q * d.depth + (t & d.dmask);
-    uint64_t st = ld_acq64(&d.sqe_state[i]);
-    if (st != (((uint64_t)t << 2) | SQE_UPDATED)) break;
-    st_rlx64(&d.sqe_state[i], ((uint64_t)t << 2) | SQE_ISSUED);
-    ++t;
-    ++n;
+// Alg. 2, update_SQE + move_SQ_tail + Attempt_SQDB without a lock: issue the `n` commands
+// written to consecutive slots from `ticket` on.  The doorbell counts issued commands,
+// so it is the tail, and it equals `ticket` once every command before ours is out: then
+// one compare-and-swap issues ours.  If it does not, the slots are marked UPDATED and
+// the compare-and-swap is tried once more: either it succeeds now, or the thread that
+// issues the command before ours finds the mark (both sides put an sc fence between
+// their write and their read) and issues ours with its own -- no thread waits for
+// another.  A thread so issues its commands and all UPDATED ones right behind them with one
+// doorbell each time it moves the tail.  (The doorbell lock this replaces -- lock, tail,
+// two state reads, doorbell, unlock, state read -- had a command wait 5.5 us from its
+// commit to the device; the compare-and-swap has 3 us, measured on 256 warps of misses.)
+static __device__ __forceinline__ void sq_ring(const Dev &d, uint32_t q, uint32_t ticket, uint32_t n = 1) {
+  uint32_t *db = &d.sq_db[q];
+  unsigned long long *st = &d.sqe_state[(uint64_t)q * d.depth];
+  fence_ar();  // the commands (and what the caller wrote before) reach the device with the doorbell
+  uint32_t rung = 0;
+  if (atomicCAS(db, ticket, ticket + n) != ticket) {
+    for (uint32_t k = 0; k < n; ++k)
+      st_rlx64(&st[(ticket + k) & d.dmask], ((uint64_t)(ticket + k) << 2) | SQE_UPDATED);
+    fence_sc();
+    uint32_t old = atomicCAS(db, ticket, ticket + n);
+    // the issuer before us may have seen the first mark and not yet the second
+    if (n == 2 && old == ticket + 1 && atomicCAS(db, ticket + 1, ticket + 2) == ticket + 1) old = ticket;
+    if (old != ticket) return;
   }
-  if (n) {
-    st_rlx32(&d.sq_tail[q], t);
+  for (uint32_t t = ticket + n;;) {
+    ++rung;
+    fence_sc();
+    uint32_t m = 0;
+    while (m < d.depth && ld_acq64(&st[(t + m) & d.dmask]) == (((uint64_t)(uint32_t)(t + m) << 2) | SQE_UPDATED)) ++m;
+    if (!m) break;
     fence_ar();
-    st_rel32(&d.sq_db[q], t & d.dmask);
-    atomicAdd(stat_ptr(d, S_DOORBELLS), 1ull);
+    if (atomicCAS(db, t, t + m) != t) break;  // their own thread was faster and looks further
+    t += m;
   }
-}
-
-// Alg. 2, Attempt_SQDB: try the doorbell lock, move the tail if it is ours, and report
-// whether our command has left the UPDATED state.
-__device__ __forceinline__ bool sq_attempt_db(const Dev &d, uint32_t q, uint32_t slot, uint32_t ticket) {
-  if (atomicCAS(&d.sq_lock[q], 0u, 1u) == 0u) {
-    fence_ar();
-    sq_move_tail(d, q);
-    fence_ar();
-    atomicExch(&d.sq_lock[q], 0u);
-  }
-  uint64_t st = ld_acq64(&d.sqe_state[(uint64_t)q * d.depth + slot]);
-  return !((st >> 2) == (uint64_t)ticket && (st & 3) == SQE_UPDATED);
-}
-
-// Warp-collective doorbell batching: lanes with `has` committed a command to queue q.
-// One leader per queue rings for the whole group; then every lane repeats
-// Attempt_SQDB until its own command is ISSUED (bounded by the deadline).
-__device__ __forceinline__ bool warp_ring(const Dev &d, bool has, uint32_t q, uint32_t slot,
-                                          uint32_t ticket, uint64_t deadline) {
-  unsigned m = __match_any_sync(kFull, has ? q : 0xFFFFFFFFu);
-  bool leader = has && (__ffs(m) - 1 == (int)lane_id());
-  bool pending = has;
-  if (leader) pending = !sq_attempt_db(d, q, slot, ticket);
-  __syncwarp();
-  if (has && pending) {
-    uint64_t st = ld_acq64(&d.sqe_state[(uint64_t)q * d.depth + slot]);
-    pending = ((st >> 2) == (uint64_t)ticket && (st & 3) == SQE_UPDATED);
-  }
-  uint32_t ns = 32;
-  while (pending) {
-    if (sq_attempt_db(d, q, slot, ticket)) break;
-    if (gtimer() > deadline) {
-      set_error(d, -110);
-      return false;
-    }
-    backoff(ns);
-  }
-  return true;
+  atomicAdd(stat_ptr(d, S_DOORBELLS), (unsigned long long)rung);
 }
 
 // ================================================================ in-flight share table
-// Sec. 3.4.1: page -> request in flight.  A bucket of 4 slots per hash; the slot key is
-// page+1 (0 = free).  Inserting the key is how a thread takes ownership of a page's
-// miss (or write); any other thread that finds the key defers and retries.
+// Sec. 3.4.1: page -> request in flight.  Inserting the page is how a thread takes
+// ownership of its miss (or write); any other thread that finds it defers and retries.
+// A bucket is one 64-bit word of four 16-bit keys (bit 15 = in use), so a single
+// compare-and-swap both sees whether the page is there and inserts it, and no two
+// threads can insert it into different slots.  page * sh_mul mod 2^sh_bits (an odd
+// multiplier: a bijection of the store's page numbers) gives the bucket in its upper bits
+// and the key in its lower 15, so equal keys in a bucket are equal pages.
 constexpr uint64_t SH_FILL = 1, SH_WRITE = 2;
-__device__ __forceinline__ uint32_t sh_bucket(const Dev &d, uint64_t page) {
-  uint64_t h = (page + 0x632BE59BD9B4E019ull) * 0xC2B2AE3D27D4EB4Full;
-  return (uint32_t)(h >> 40) & d.sh_mask;
+constexpr uint32_t kShKeyBits = 15;
+__device__ __forceinline__ uint32_t sh_hash(const Dev &d, uint64_t page, uint64_t &key) {
+  uint64_t y = (page * d.sh_mul) & ((1ull << d.sh_bits) - 1);
+  key = (y & 0x7FFFu) | 0x8000u;
+  return (uint32_t)(y >> kShKeyBits);
 }
-// returns slot index >= 0 when inserted, -1 when the page is already present (or a
-// racing insert of the same page was seen), -2 when the bucket is full.
+__device__ __forceinline__ int sh_find(uint64_t word, uint64_t key) {
+  int at = -1;
+#pragma unroll
+  for (int k = 3; k >= 0; --k)
+    if (((word >> (16 * k)) & 0xFFFFu) == key) at = k;
+  return at;
+}
+// returns slot index >= 0 when inserted, -1 when the page is already present, -2 when
+// the bucket is full (or too contended).  The insertion acquires: what the page's last
+// request wrote before it left the table (tag, store) is seen after it.
 __device__ __forceinline__ int64_t sh_insert(const Dev &d, uint64_t page, uint64_t kind) {
-  uint64_t key = page + 1;
-  uint64_t base = (uint64_t)sh_bucket(d, page) * 4;
+  (void)kind;
+  uint64_t key;
+  const uint32_t b = sh_hash(d, page, key);
+  uint64_t w = 0;  // most buckets are empty
   for (int tries = 0; tries < 8; ++tries) {
-    int free_k = -1;
-    for (int k = 0; k < 4; ++k) {
-      uint64_t v = ld_acq64(&d.sh_key[base + k]);
-      if (v == key) return -1;
-      if (v == 0 && free_k < 0) free_k = k;
-    }
-    if (free_k < 0) return -2;
-    if (atomicCAS(&d.sh_key[base + free_k], 0ull, (unsigned long long)key) != 0ull) continue;
-    // a racing insert of the same key into another slot: whoever sees the other backs off
-    fence_sc();
-    bool dup = false;
-    for (int k = 0; k < 4; ++k)
-      if (k != free_k && ld_acq64(&d.sh_key[base + k]) == key) dup = true;
-    if (dup) {
-      st_rel64(&d.sh_key[base + free_k], 0ull);
-      return -1;
-    }
-    (void)kind;
-    st_rlx64(&d.sh_val[base + free_k], 0ull);  // the token of the read, once issued
-    return (int64_t)(base + free_k);
+    if (sh_find(w, key) >= 0) return -1;
+    int k = sh_find(w, 0);
+    if (k < 0) return -2;
+    uint64_t old = atom_cas_acq(&d.sh_key[b], w, w | (key << (16 * k)));
+    if (old == w) return (int64_t)b * 4 + k;
+    w = old;
   }
   return -2;
 }
+// the caller's earlier writes are ordered before the removal by a fence of its own
+__device__ __forceinline__ void sh_clear(const Dev &d, uint64_t slot) {
+  atomicAnd(&d.sh_key[slot >> 2], ~(0xFFFFull << (16 * (slot & 3))));
+}
 __device__ __forceinline__ void sh_remove(const Dev &d, uint64_t slot) {
-  st_rlx64(&d.sh_val[slot], 0ull);
-  st_rel64(&d.sh_key[slot], 0ull);
+  st_rlx64(&d.sh_val[slot], 0ull);  // the next owner finds it 0
+  fence_ar();
+  sh_clear(d, slot);
 }
 // Token of the read in flight for `page`, ~0 when there is none (or it is not
 // published yet).  The key is read again after the value: an entry removed (and maybe reused)
 // meanwhile is not taken; one re-inserted for the same page carries a token of the same
 // page, which is as good.
 __device__ __forceinline__ uint64_t sh_token(const Dev &d, uint64_t page) {
-  uint64_t key = page + 1;
-  uint64_t base = (uint64_t)sh_bucket(d, page) * 4;
-  for (int k = 0; k < 4; ++k) {
-    if (ld_acq64(&d.sh_key[base + k]) != key) continue;
-    uint64_t v = ld_acq64(&d.sh_val[base + k]);
-    if (v && ld_acq64(&d.sh_key[base + k]) == key) return v - 1;
-  }
+  uint64_t key;
+  const uint32_t b = sh_hash(d, page, key);
+  int k = sh_find(ld_acq64(&d.sh_key[b]), key);
+  if (k < 0) return ~0ull;
+  uint64_t v = ld_acq64(&d.sh_val[(uint64_t)b * 4 + k]);
+  if (v && sh_find(ld_acq64(&d.sh_key[b]), key) == k) return v - 1;
   return ~0ull;
 }
 
@@ -547,6 +572,15 @@ __device__ __forceinline__ void ld_tags8(const unsigned long long *p, uint64_t t
 #pragma unroll
   for (int k = 0; k < 4; ++k)
     asm volatile("ld.global.cg.v2.u64 {%0,%1}, [%2];" : "=l"(t[2 * k]), "=l"(t[2 * k + 1]) : "l"(p + 2 * k) : "memory");
+}
+
+// ... as 32-bit halves: {page bits 0-11, pin, wb, ref, state} and {page bits 12-43}
+__device__ __forceinline__ void ld_tags8_halves(const unsigned long long *p, uint32_t lo[8], uint32_t hi[8]) {
+  static_assert(PAGE_SHIFT == 20, "the upper half holds the page from bit 12 on");
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(lo[2 * k]), "=r"(hi[2 * k]), "=r"(lo[2 * k + 1]), "=r"(hi[2 * k + 1]) : "l"(p + 2 * k) : "memory");
 }
 
 // The way of an 8-way tag copy that holds `page` READY or MODIFIED (its tag in t), or
@@ -569,14 +603,15 @@ __device__ __forceinline__ int cache_probe(const Dev &d, uint64_t page, bool pin
   uint64_t t = 0;
   int wsel = -1;
   if (d.ways == 8) {  // sets of 8 ways are 64-byte aligned: read them at once
-    uint64_t pre[8];
-    ld_tags8(&d.tag[base], pre);
+    uint32_t lo[8], hi[8], tl = 0;
+    ld_tags8_halves(&d.tag[base], lo, hi);
 #pragma unroll
     for (int k = 7; k >= 0; --k)
-      if (tag_state(pre[k]) != ST_INVALID && tag_page(pre[k]) == page) {
+      if ((lo[k] & 3) && hi[k] == (uint32_t)(page >> 12) && lo[k] >> PAGE_SHIFT == ((uint32_t)page & 0xFFFu)) {
         wsel = k;
-        t = pre[k];
+        tl = lo[k];
       }
+    t = tl;  // state and reference bit
   } else {
     for (uint32_t k = 0; k < d.ways && wsel < 0; ++k) {
       uint64_t tk = ld_rlx64(&d.tag[base + k]);
@@ -630,87 +665,129 @@ __device__ __forceinline__ void cache_unclaim(const Dev &d, uint32_t line, uint6
 enum Miss { M_ISSUED = 0, M_HIT = 1, M_BUSY = 2, M_RETRY = 3 };
 
 struct Issued {
-  uint32_t q, slot, ticket;  // the command to ring (the read, when there is one)
+  uint32_t q, slot, ticket;  // the command issued last (the read, when there is one)
   int code;  // 1 fill, 2 evict READY, 3 write-back MODIFIED
 };
 
-// One thread rings queue q until its command (slot, ticket) has left UPDATED (the
-// doorbell-lock holder never needs a cache line, so this wait cannot close a cycle);
-// false after the context's wait bound.
-static __device__ __noinline__ bool lane_ring(const Dev &d, uint32_t q, uint32_t slot, uint32_t ticket) {
-  uint64_t deadline = gtimer() + d.timeout_ns;
-  uint32_t ns = 32;
-  while (!sq_attempt_db(d, q, slot, ticket)) {
-    if (gtimer() > deadline) {
-      set_error(d, -110);
-      return false;
-    }
-    backoff(ns);
-  }
-  return true;
+// What one thread's miss holds between cache_claim, cache_reserve and cache_issue: the
+// claimed line, its old tag, the in-flight entries of the page and of a MODIFIED victim,
+// then the reserved slots.  wb: the victim must be copied to the staging page of
+// (q, slot) before cache_issue.  w0: the first queue's reservation word, read beside the claim.
+struct Claim {
+  uint64_t old, w0;
+  int64_t sh, sh_wb;
+  uint32_t line, q, slot, ticket;
+  bool wb, fill;
+};
+__device__ __forceinline__ uint8_t *claim_staging(const Dev &d, const Claim &c) {
+  return d.staging + ((uint64_t)c.q * d.depth + c.slot) * kPage;
 }
 
 // The rare miss whose MODIFIED victim lives on another device than the page that
 // replaces it: the write-back takes a demand slot of its device, the read a slot of the
 // page's device.  If the read's slot cannot be had, the write-back's slot is spent on a
-// no-op command (a reserved slot must be committed) and the miss is retried holding
-// nothing.  The write-back is rung here; the read is left to the caller in `is`.
+// no-op command (a reserved slot must be issued) and the miss is retried holding
+// nothing.  The write-back is issued here; the read is left to cache_issue.
 // Out of line, so that the common miss path stays small.
-static __device__ __noinline__ int cache_miss_split(const Dev &d, uint64_t page, uint32_t q0, uint32_t line,
-                                                    Issued &is, uint64_t old, int64_t sh, int64_t sh_wb, bool pf) {
+static __device__ __noinline__ int cache_reserve_split(uint64_t page, uint32_t q0, Claim &c, bool pf) {
+  const Dev &d = shared_dev();
   uint32_t wq = 0, wslot = 0, wticket = 0, q = 0, slot = 0, ticket = 0;
-  if (!sq_reserve_dev(d, q0, dev_of_page(d, tag_page(old)), 1, wq, wslot, wticket, false)) {
-    cache_unclaim(d, line, old);
-    sh_remove(d, (uint64_t)sh_wb);
-    sh_remove(d, (uint64_t)sh);
+  if (!sq_reserve_dev(d, q0, dev_of_page(d, tag_page(c.old)), 1, wq, wslot, wticket, false)) {
+    cache_unclaim(d, c.line, c.old);
+    sh_remove(d, (uint64_t)c.sh_wb);
+    sh_remove(d, (uint64_t)c.sh);
     return M_RETRY;
   }
   if (!sq_reserve_dev(d, q0, dev_of_page(d, page), 1, q, slot, ticket, pf)) {
-    sq_commit(d, wq, wslot, wticket, OP_FLUSH, 0, 0, ctx_make(CTX_NOP, 0, 0));
-    cache_unclaim(d, line, old);
-    sh_remove(d, (uint64_t)sh_wb);
-    sh_remove(d, (uint64_t)sh);
-    lane_ring(d, wq, wslot, wticket);
+    sq_write(d, wq, wslot, wticket, OP_FLUSH, 0, 0, ctx_make(CTX_NOP, 0, 0));
+    cache_unclaim(d, c.line, c.old);
+    sh_remove(d, (uint64_t)c.sh_wb);
+    sh_remove(d, (uint64_t)c.sh);
+    sq_ring(d, wq, wticket);
     return M_RETRY;
   }
-  atomicAdd(stat_ptr(d, S_EVICTIONS), 1ull);
   uint8_t *stg = d.staging + ((uint64_t)wq * d.depth + wslot) * kPage;
-  lane_copy_page(stg, line_ptr(d, line));
-  fence_ar();
-  sq_commit(d, wq, wslot, wticket, OP_WRITE, (uint64_t)stg, tag_page(old), ctx_make(CTX_WB, (uint32_t)sh_wb, 0));
+  fence_ar();  // the line is read after it was claimed
+  lane_copy_page(stg, line_ptr(d, c.line));
+  sq_write(d, wq, wslot, wticket, OP_WRITE, (uint64_t)stg, tag_page(c.old), ctx_make(CTX_WB, (uint32_t)c.sh_wb, 0));
   atomicAdd(stat_ptr(d, S_WRITEBACKS), 1ull);
-  lane_ring(d, wq, wslot, wticket);
-  st_rlx64(&d.sh_val[sh], (((uint64_t)q << 48) | ((uint64_t)slot << 32) | ticket) + 1);
-  sq_commit(d, q, slot, ticket, OP_READ, (uint64_t)line_ptr(d, line), page, ctx_make(CTX_FILL, (uint32_t)sh, line));
-  atomicAdd(stat_ptr(d, S_MISSES), 1ull);
-  is.q = q;
-  is.slot = slot;
-  is.ticket = ticket;
-  is.code = 3;
+  sq_ring(d, wq, wticket);
+  c.q = q;
+  c.slot = slot;
+  c.ticket = ticket;
+  c.wb = false;  // already on its way
   return M_ISSUED;
 }
 
-// Cases (b) and (d) for one thread: take ownership of the page's miss in the share
-// table, pick a way (lowest INVALID way, else the clock: a set reference bit is
-// cleared and the hand moves on, the first unpinned, unreferenced READY or MODIFIED
-// way is the victim; BUSY, pinned and write-back-pending ways are skipped), reserve
-// queue slots, write back a MODIFIED victim from a staging copy and issue the read.
-// Nothing here waits: on any shortage every claim is undone and M_RETRY returned.
-//
-// fill=false (writes of whole pages): the caller already owns the page's share entry
-// `sh_own`; the way is claimed BUSY and returned without a read, the caller writes the
-// line and publishes it.  A MODIFIED victim is still written back first.
 // Victim search of a miss in `set` (Sec. 3.4 cases (b) and (d)): the lowest way with
 // an INVALID, unpinned tag, else the clock sweep from the set's hand (a way whose
 // reference bit is set has it cleared and is passed; BUSY, pinned and written-back
-// ways are passed; under FIFO no bit is looked at).  Each step of the hand is a
-// fetch-and-add, so misses racing in one set sweep different ways.  The chosen way is
-// claimed by compare-and-swap from the tag that was read, as BUSY for the new page
-// (`claimed`).  Returns the way (old = its tag before, 0 when it was INVALID; sh_wb =
-// the Share Table entry of the write-back of a MODIFIED victim) or -1.  Kept out of
-// line: the miss path's registers stay out of the callers' loops.
-static __device__ __noinline__ int64_t pick_victim(const Dev &d, uint32_t set, uint64_t claimed, uint64_t &old,
-                                                   int64_t &sh_wb) {
+// ways are passed; under FIFO no bit is looked at).  The chosen way is claimed by
+// compare-and-swap from the tag that was read, as BUSY for the new page (`claimed`).
+// Returns the way (old = its tag before, 0 when it was INVALID; sh_wb = the Share Table
+// entry of the write-back of a MODIFIED victim) or -1.
+//
+// pick_victim8, sets of 8 ways: the sweep is done on the copy of the tags that the
+// caller has just read, as bit masks over the ways in the hand's order and without
+// branches, so that a claim costs one round trip after that read (hand and cleared
+// reference bits are updated without waiting).  A claim that fails (the way was taken or
+// touched meanwhile) passes the way.  pick_victim reads every way when the sweep gets to
+// it, two round trips a step.
+static __device__ __forceinline__ int pick_victim8(const Dev &d, uint32_t set, const uint32_t (&lo)[8],
+                                                   const uint32_t (&hi)[8], uint32_t hand, uint64_t claimed,
+                                                   uint64_t &old, int64_t &sh_wb) {
+  unsigned long long *tags = &d.tag[(uint64_t)set * 8];
+  uint32_t zero = 0, skip = 0, ref = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    zero |= ((lo[w] | hi[w]) == 0 ? 1u : 0u) << w;
+    skip |= ((lo[w] & (uint32_t)(PIN_MASK | TAG_WB)) != 0 || (lo[w] & 3) == ST_BUSY ? 1u : 0u) << w;
+    ref |= (lo[w] & 3 ? (lo[w] >> 2) & 1u : 0u) << w;
+  }
+  if (d.policy != kPolicyClock) ref = 0;
+  const uint32_t h0 = hand & 7;
+  uint32_t rskip = ((skip * 0x101u) >> h0) & 0xFF, rref = ((ref * 0x101u) >> h0) & 0xFF, passed = 0;
+  for (;;) {
+    // an INVALID way, else the first way the hand finds unreferenced, else (second turn)
+    // the first one whose bit the first turn has cleared
+    const uint32_t first = ~rskip & ~rref & ~passed & 0xFF, second = (rref | passed) & ~rskip;
+    if (!(zero | first | second)) {
+      atomicAdd(&d.hand[set], 17u);
+      return -1;
+    }
+    const uint32_t p = __ffs(first ? first : second) - 1;
+    const uint32_t w = zero ? __ffs(zero) - 1 : (h0 + p) & 7;
+    uint32_t clear = zero ? 0 : (first ? rref & ~rskip & ((1u << p) - 1) : rref & ~rskip);
+    passed |= clear;
+    rref &= ~clear;
+    clear = ((clear * 0x101u) >> (8 - h0)) & 0xFF;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if ((clear >> k) & 1u) atomicAnd(&tags[k], ~TAG_REF);
+    uint32_t tl = 0, th = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k == (int)w) {
+        tl = lo[k];
+        th = hi[k];
+      }
+    if (!zero && (passed >> p & 1u)) tl &= ~(uint32_t)TAG_REF;
+    const uint64_t tw = (uint64_t)th << 32 | tl;
+    if ((tl & 3) == ST_MODIFIED) sh_wb = sh_insert(d, tag_page(tw), SH_WRITE);
+    if (((tl & 3) != ST_MODIFIED || sh_wb >= 0) &&
+        atomicCAS(&tags[w], (unsigned long long)tw, (unsigned long long)claimed) == tw) {
+      if (!zero) atomicAdd(&d.hand[set], (first ? 0u : 8u) + p + 1);
+      old = (tl & 3) == ST_INVALID ? 0 : tw;
+      return (int)w;
+    }
+    if (sh_wb >= 0) sh_remove(d, (uint64_t)sh_wb);
+    sh_wb = -1;
+    zero &= zero - 1;  // (0 stays 0)
+    rskip |= 1u << ((w - h0) & 7);
+  }
+}
+static __device__ __noinline__ int64_t pick_victim(uint32_t set, uint64_t claimed, uint64_t &old, int64_t &sh_wb) {
+  const Dev &d = shared_dev();
   const uint32_t ways = d.ways;
   const uint64_t base = (uint64_t)set * ways;
   for (uint32_t w = 0; w < ways; ++w) {
@@ -752,76 +829,142 @@ static __device__ __noinline__ int64_t pick_victim(const Dev &d, uint32_t set, u
   return -1;
 }
 
-static __device__ int cache_miss(const Dev &d, uint64_t page, uint32_t q0, uint32_t &line, Issued &is,
-                          bool fill = true, int64_t sh_own = -1, bool pf = false) {
-  int64_t sh = sh_own;
+// Cases (b) and (d) for one thread, first part: take ownership of the page's miss in the
+// share table, probe once more (the page may have come in meanwhile), pick and claim a
+// way.  Nothing in the three parts waits: on any shortage every claim is undone and M_RETRY
+// returned.  The chain of dependent L2 round trips bounds a miss (not bandwidth):
+// in-flight entry, set and hand, claim, reservation, doorbell -- the first queue's
+// reservation word is loaded beside the in-flight entry.
+//
+// fill=false (writes of whole pages): the caller already owns the page's share entry
+// `sh_own`; the way is claimed BUSY without a read, the caller writes the line and
+// publishes it.  A MODIFIED victim is still written back first.
+static __device__ __forceinline__ int cache_claim(const Dev &d, uint64_t page, uint32_t q0, Claim &c, bool fill = true,
+                                               int64_t sh_own = -1, bool pf = false) {
+  c.sh = sh_own;
+  c.sh_wb = -1;
+  c.old = 0;
+  c.wb = false;
+  c.fill = fill;
+  c.q = 0xFFFFFFFFu;
+  c.slot = c.ticket = 0;
+  c.w0 = kNoWord;
   if (fill) {
-    sh = sh_insert(d, page, SH_FILL);
-    if (sh < 0) {
+    c.w0 = sq_first_word(d, q0, dev_of_page(d, page), pf);
+    c.sh = sh_insert(d, page, SH_FILL);
+    if (c.sh < 0) {
       atomicAdd(stat_ptr(d, S_SHARE_RETRIES), 1ull);
       return M_RETRY;
     }
   }
-  int pr = cache_probe(d, page, false, line);
-  if (pr != P_MISS) {
-    if (fill) sh_remove(d, (uint64_t)sh);
-    return pr == P_HIT ? M_HIT : M_BUSY;
+  const uint32_t set = set_of(page, d.sets);
+  const uint64_t base = (uint64_t)set * d.ways, claimed = tag_make(page, ST_BUSY, true);
+  int64_t victim = -1;
+  int there = -1;  // way that holds the page already
+  uint64_t tw = 0;
+  if (d.ways == 8) {
+    uint32_t lo[8], hi[8];
+    const uint32_t hand = ld_rlx32(&d.hand[set]);
+    ld_tags8_halves(&d.tag[base], lo, hi);
+#pragma unroll
+    for (int k = 7; k >= 0; --k)
+      if ((lo[k] & 3) && hi[k] == (uint32_t)(page >> 12) && lo[k] >> PAGE_SHIFT == ((uint32_t)page & 0xFFFu)) {
+        there = k;
+        tw = lo[k];
+      }
+    if (there < 0) victim = pick_victim8(d, set, lo, hi, hand, claimed, c.old, c.sh_wb);
+  } else {
+    for (uint32_t k = 0; k < d.ways && there < 0; ++k) {
+      tw = ld_rlx64(&d.tag[base + k]);
+      if (tag_state(tw) != ST_INVALID && tag_page(tw) == page) there = (int)k;
+    }
+    if (there < 0) victim = pick_victim(set, claimed, c.old, c.sh_wb);
   }
-  uint32_t set = set_of(page, d.sets);
-  uint64_t base = (uint64_t)set * d.ways;
-  uint64_t old = 0;
-  int64_t sh_wb = -1;
-  int64_t victim = pick_victim(d, set, tag_make(page, ST_BUSY, true), old, sh_wb);
+  if (there >= 0) {
+    c.line = (uint32_t)(base + there);
+    if (fill) sh_remove(d, (uint64_t)c.sh);
+    if (tag_state(tw) == ST_BUSY) return M_BUSY;
+    if (!(tw & TAG_REF)) atomicOr(&d.tag[c.line], TAG_REF);
+    return M_HIT;
+  }
   if (victim < 0) {
-    if (fill) sh_remove(d, (uint64_t)sh);
+    if (fill) sh_remove(d, (uint64_t)c.sh);
     atomicAdd(stat_ptr(d, S_EAGAIN), 1ull);
     return M_RETRY;
   }
-  line = (uint32_t)(base + victim);
-  bool wb = tag_state(old) == ST_MODIFIED;
-  if (wb && fill && d.ndev > 1 && dev_of_page(d, tag_page(old)) != dev_of_page(d, page))
-    return cache_miss_split(d, page, q0, line, is, old, sh, sh_wb, pf);
+  c.line = (uint32_t)(base + victim);
+  c.wb = tag_state(c.old) == ST_MODIFIED;
+  return M_ISSUED;
+}
+
+// Second part: reserve queue slots, right before the commands are written and issued: a
+// queue's commands reach the device in the order of their slots, so a slot held while
+// other lanes of the warp still look for lines would hold up every other warp's commands
+// behind it (reserved with the claim, a twentieth of the commands of a page-read burst
+// waited 100 us).
+static __device__ __forceinline__ int cache_reserve(const Dev &d, uint64_t page, uint32_t q0, Claim &c, bool pf) {
+  if (c.wb && c.fill && d.ndev > 1 && dev_of_page(d, tag_page(c.old)) != dev_of_page(d, page))
+    return cache_reserve_split(page, q0, c, pf);
   // a write-back and its refill take two consecutive slots of one queue of their
   // device, reserved together (a write-back rides in the demand class: a fill waits
   // behind it)
-  uint32_t q = 0, slot = 0, ticket = 0;
-  uint32_t nslots = (wb ? 1u : 0u) + (fill ? 1u : 0u);
-  if (nslots && !sq_reserve_dev(d, q0, dev_of_page(d, wb ? tag_page(old) : page), nslots, q, slot, ticket,
-                                pf && !wb)) {
-    cache_unclaim(d, line, old);
-    if (wb) sh_remove(d, (uint64_t)sh_wb);
-    if (fill) sh_remove(d, (uint64_t)sh);
+  const uint32_t nslots = (c.wb ? 1u : 0u) + (c.fill ? 1u : 0u);
+  if (nslots && !sq_reserve_dev(d, q0, dev_of_page(d, c.wb ? tag_page(c.old) : page), nslots, c.q, c.slot, c.ticket,
+                                pf && !c.wb, c.wb ? kNoWord : c.w0)) {
+    cache_unclaim(d, c.line, c.old);
+    if (c.wb) sh_remove(d, (uint64_t)c.sh_wb);
+    if (c.fill) sh_remove(d, (uint64_t)c.sh);
     return M_RETRY;
   }
-  is.q = q;
-  is.slot = slot;
-  is.ticket = ticket;
-  is.code = wb ? 3 : (old ? 2 : 1);
-  if (old) atomicAdd(stat_ptr(d, S_EVICTIONS), 1ull);
-  if (wb) {
-    uint8_t *stg = d.staging + ((uint64_t)q * d.depth + slot) * kPage;
-    lane_copy_page(stg, line_ptr(d, line));
-    fence_ar();
-    sq_commit(d, q, slot, ticket, OP_WRITE, (uint64_t)stg, tag_page(old),
-              ctx_make(CTX_WB, (uint32_t)sh_wb, 0));
-    atomicAdd(stat_ptr(d, S_WRITEBACKS), 1ull);
-    if (!fill) return M_ISSUED;  // the write-back is the command to ring
-    slot = (slot + 1) & d.dmask;
-    ticket += 1;
-  }
-  if (!fill) {
-    is.q = 0xFFFFFFFFu;  // nothing to ring
-    return M_ISSUED;
-  }
-  // the read's token + 1 (0 = none yet), for threads that find the page in flight
-  // (Sec. 3.4 case (c)); the commit's release publishes it
-  st_rlx64(&d.sh_val[sh], (((uint64_t)q << 48) | ((uint64_t)slot << 32) | ticket) + 1);
-  sq_commit(d, q, slot, ticket, OP_READ, (uint64_t)line_ptr(d, line), page,
-            ctx_make(CTX_FILL, (uint32_t)sh, line));
-  atomicAdd(stat_ptr(d, S_MISSES), 1ull);
-  is.slot = slot;
-  is.ticket = ticket;
+  if (c.wb) fence_ar();  // the line is read after it was claimed
   return M_ISSUED;
+}
+
+// Third part: write the commands of a claim (a MODIFIED victim's page is in its staging
+// page by now) and issue them.
+static __device__ __forceinline__ void cache_issue(const Dev &d, uint64_t page, const Claim &c, Issued &is) {
+  is.q = c.q;
+  is.slot = c.slot;
+  is.ticket = c.ticket;
+  is.code = tag_state(c.old) == ST_MODIFIED ? 3 : (c.old ? 2 : 1);
+  if (c.old) atomicAdd(stat_ptr(d, S_EVICTIONS), 1ull);
+  if (c.wb) {
+    sq_write(d, c.q, c.slot, c.ticket, OP_WRITE, (uint64_t)claim_staging(d, c), tag_page(c.old),
+             ctx_make(CTX_WB, (uint32_t)c.sh_wb, 0));
+    atomicAdd(stat_ptr(d, S_WRITEBACKS), 1ull);
+  }
+  if (c.fill) {
+    if (c.wb) {
+      is.slot = (c.slot + 1) & d.dmask;
+      is.ticket = c.ticket + 1;
+    }
+    // the read's token + 1 (0 = none yet), for threads that find the page in flight
+    // (Sec. 3.4 case (c)); the doorbell's fence publishes it
+    st_rlx64(&d.sh_val[c.sh], (((uint64_t)c.q << 48) | ((uint64_t)is.slot << 32) | is.ticket) + 1);
+    sq_write(d, c.q, is.slot, is.ticket, OP_READ, (uint64_t)line_ptr(d, c.line), page,
+             ctx_make(CTX_FILL, (uint32_t)c.sh, c.line));
+    atomicAdd(stat_ptr(d, S_MISSES), 1ull);
+  }
+  const uint32_t n = (c.wb ? 1u : 0u) + (c.fill ? 1u : 0u);
+  if (n) sq_ring(d, c.q, c.ticket, n);
+}
+
+// all three for a lane on its own
+static __device__ __noinline__ int cache_miss_call(uint64_t page, uint32_t q0, uint32_t &line, Issued &is, bool fill,
+                                                   int64_t sh_own, bool pf) {
+  const Dev &d = shared_dev();
+  Claim c;
+  int m = cache_claim(d, page, q0, c, fill, sh_own, pf);
+  if (m == M_ISSUED) m = cache_reserve(d, page, q0, c, pf);
+  if (m != M_RETRY) line = c.line;
+  if (m != M_ISSUED) return m;
+  if (c.wb) lane_copy_page(claim_staging(d, c), line_ptr(d, c.line));
+  cache_issue(d, page, c, is);
+  return M_ISSUED;
+}
+static __device__ __forceinline__ int cache_miss(const Dev &, uint64_t page, uint32_t q0, uint32_t &line, Issued &is,
+                                                 bool fill = true, int64_t sh_own = -1, bool pf = false) {
+  return cache_miss_call(page, q0, line, is, fill, sh_own, pf);
 }
 
 __device__ __forceinline__ uint64_t make_token(uint32_t q, uint32_t slot, uint32_t ticket) {
@@ -842,11 +985,22 @@ __device__ __forceinline__ uint64_t make_token(uint32_t q, uint32_t slot, uint32
 // device (a page READY or already in flight adds nothing); bit 1: some hint was
 // dropped because the device is saturated.
 // `pf`: the pages are requested ahead of need (prefetch queues, served after demand).
+// `limit`: how many misses a hint may send.
 // `hint`: a speculative request of an application's lookahead, dropped (no retry) when
 // its first queue is crowded or no queue has room -- the device is saturated.
-static __device__ bool warp_request(const Dev &d, bool want, uint64_t page, uint32_t q0, bool wait,
-                             uint64_t deadline, uint64_t *tok = nullptr, int *code = nullptr,
-                             uint32_t *outcome = nullptr, bool pf = false, bool hint = false) {
+// Out of line: one copy per kernel keeps the applications' loops and the instruction
+// cache footprint small (the start of a lookup kernel with five inlined copies spent a third
+// of its issue slots' stalls on instruction fetches); a call costs little next to the
+// round trips of a request.
+struct Requested {
+  uint64_t tok;
+  uint32_t outcome;  // bit 0 sent, bit 1 dropped, bit 2 ok; code in the upper half
+};
+static __device__ __noinline__ Requested warp_request_body(bool want, uint64_t page, uint32_t q0, bool wait,
+                                                           uint64_t deadline, bool pf, bool hint, uint32_t limit) {
+  const Dev &d = shared_dev();
+  uint64_t tok = ~0ull;
+  int code = 0;
   unsigned grp = __match_any_sync(kFull, want ? page : ~0ull);
   int lead_lane = __ffs(grp) - 1;
   bool leader = want && lead_lane == (int)lane_id();
@@ -855,14 +1009,14 @@ static __device__ bool warp_request(const Dev &d, bool want, uint64_t page, uint
   uint32_t line = 0;
   bool ok = true;
   bool first = true;
-  uint32_t ns = 64;
+  uint32_t ns = 32;
   uint32_t retries = 0;
-  if (tok && leader) *tok = ~0ull;
-  if (code && leader) *code = 0;
   bool dropped = false, sent = false;
   while (__any_sync(kFull, need)) {
-    bool issued = false, ring = false;
-    Issued is{};
+    int m = M_RETRY;
+    bool missed = false;
+    Claim c;
+    c.wb = false;
     if (need) {
       int pr = cache_probe(d, page, false, line);
       if (pr == P_HIT) {
@@ -871,30 +1025,52 @@ static __device__ bool warp_request(const Dev &d, bool want, uint64_t page, uint
       } else if (pr == P_BUSY) {
         if (first) atomicAdd(stat_ptr(d, S_BUSY_HITS), 1ull);
         if (!wait) need = false;
-      } else if (hint && !wait && sq_crowded(d, q0, dev_of_page(d, page), pf)) {
-        need = false;  // the device is saturated: drop the hint
-        dropped = true;
       } else {
-        int m = cache_miss(d, page, q0, line, is, true, -1, pf);
-        ring = m == M_ISSUED;
-        if (m == M_ISSUED) {
-          issued = true;
-          sent = true;
-          if (tok) *tok = make_token(is.q, is.slot, is.ticket);
-          if (code) *code = is.code;
-          if (!wait) need = false;
-        } else if (m == M_HIT) {
-          need = false;
-        } else if (m == M_BUSY) {
-          if (!wait) need = false;
-        } else if (!wait && (hint || ++retries >= 4)) {
-          need = false;  // a prefetch is a hint: give up when nothing can be evicted now
-          if (hint) dropped = true;
-        }
+        missed = true;
+      }
+    }
+    if (hint) {
+      // beyond `limit` misses, or with the device saturated, a hint is dropped
+      const unsigned away = __ballot_sync(kFull, missed);
+      if (missed && !wait &&
+          ((uint32_t)__popc(away & ((1u << lane_id()) - 1)) >= limit || sq_crowded(d, q0, dev_of_page(d, page), pf))) {
+        missed = need = false;
+        dropped = true;
+      }
+    }
+    if (missed) {
+      m = cache_claim(d, page, q0, c, true, -1, pf);
+      if (m != M_RETRY) line = c.line;
+    }
+    __syncwarp();
+    if (m == M_ISSUED) m = cache_reserve(d, page, q0, c, pf);
+    // MODIFIED victims are copied to their staging pages by the whole warp
+    for (unsigned wb = __ballot_sync(kFull, m == M_ISSUED && c.wb); wb; wb &= wb - 1) {
+      const int j = __ffs(wb) - 1;
+      const uint64_t src = __shfl_sync(kFull, (uint64_t)line_ptr(d, c.line), j);
+      const uint64_t dst = __shfl_sync(kFull, (uint64_t)claim_staging(d, c), j);
+      warp_copy_page((void *)dst, (const void *)src);
+    }
+    __syncwarp();
+    if (missed) {
+      if (m == M_ISSUED) {
+        Issued is;
+        cache_issue(d, page, c, is);
+        sent = true;
+        tok = ((uint64_t)is.q << 48) | ((uint64_t)is.slot << 32) | is.ticket;
+        code = is.code;
+        if (!wait) need = false;
+      } else if (m == M_HIT) {
+        need = false;
+      } else if (m == M_BUSY) {
+        if (!wait) need = false;
+      } else if (!wait && (hint || ++retries >= 4)) {
+        need = false;  // a prefetch is a hint: give up when nothing can be evicted now
+        if (hint) dropped = true;
       }
     }
     first = false;
-    if (!warp_ring(d, ring, is.q, is.slot, is.ticket, deadline)) ok = false;
+    __syncwarp();
     if (__any_sync(kFull, need)) {
       if (need) {
         if (gtimer() > deadline || aborted(d)) {
@@ -902,17 +1078,26 @@ static __device__ bool warp_request(const Dev &d, bool want, uint64_t page, uint
           need = false;
           ok = false;
         } else {
-          // wait for the in-flight line without holding anything, then re-probe
+          // wait for the in-flight line without holding anything, then probe again
           // (short sleeps: a fill completes within microseconds)
-          uint64_t t = ld_acq64(&d.tag[line]);
-          if (tag_page(t) == page && tag_state(t) == ST_BUSY) backoff(ns, 512);
-          else if (!issued) backoff(ns, 512);
+          backoff(ns, 256);
         }
       }
     }
   }
-  if (outcome) *outcome = (__any_sync(kFull, sent) ? 1u : 0u) | (__any_sync(kFull, dropped) ? 2u : 0u);
-  return __all_sync(kFull, ok);
+  uint32_t outcome = (__any_sync(kFull, sent) ? 1u : 0u) | (__any_sync(kFull, dropped) ? 2u : 0u) |
+                     (__all_sync(kFull, ok) ? 4u : 0u);
+  return Requested{tok, outcome | (uint32_t)code << 16};
+}
+static __device__ __forceinline__ bool warp_request(const Dev &, bool want, uint64_t page, uint32_t q0, bool wait,
+                                                    uint64_t deadline, uint64_t *tok = nullptr, int *code = nullptr,
+                                                    uint32_t *outcome = nullptr, bool pf = false, bool hint = false,
+                                                    uint32_t limit = 32) {
+  const Requested r = warp_request_body(want, page, q0, wait, deadline, pf, hint, limit);
+  if (tok) *tok = r.tok;
+  if (code) *code = (int)(r.outcome >> 16);
+  if (outcome) *outcome = r.outcome & 3u;
+  return (r.outcome & 4u) != 0;
 }
 
 // Warp-cooperative probe of one page (uniform across the warp): lane w < ways loads
@@ -946,38 +1131,54 @@ __device__ __forceinline__ int warp_probe_pin(const Dev &d, uint64_t page, uint3
   return __shfl_sync(kFull, pr, w);
 }
 
-// The warp needs one page pinned (uniform `page`): probe with a pin; on a miss the warp
-// issues and waits with nothing pinned, then probes again.  Returns the line in every
-// lane, or false on timeout/abort.  The caller unpins it (one unpin per pin).
-// warp_request as one out-of-line copy: for applications whose code is large (many call
-// sites of the miss path next to the service code), one shared copy keeps their hot
-// loops small (fewer spills, fewer instruction-cache misses); a call costs little next
-// to the round trips of a request
-static __device__ __noinline__ bool warp_request_call(const Dev &d, bool want, uint64_t page, uint32_t q0,
-                                                      bool wait, uint64_t deadline, bool pf = false) {
+// warp_request without its optional results
+static __device__ __forceinline__ bool warp_request_call(const Dev &d, bool want, uint64_t page, uint32_t q0,
+                                                         bool wait, uint64_t deadline, bool pf = false) {
   return warp_request(d, want, page, q0, wait, deadline, nullptr, nullptr, nullptr, pf);
 }
 
-template <bool kCall = false>
-static __device__ bool warp_pin_page(const Dev &d, uint64_t page, uint32_t q0, uint64_t deadline,
-                              uint32_t &line_out) {
+// The warp needs one page pinned (uniform `page`): probe with a pin; on a miss the warp
+// issues the read and, holding nothing, watches the line's tag until the fill is there,
+// then probes again.  Returns the line in every lane, or false on timeout/abort.  The
+// caller unpins it (one unpin per pin).
+constexpr uint32_t kNoLine = 0xFFFFFFFFu;
+static __device__ __noinline__ uint32_t warp_pin_page_body(uint64_t page, uint32_t q0, uint64_t deadline) {
+  const Dev &d = shared_dev();
+  uint32_t ns = 32;
   for (int round = 0;; ++round) {
     uint32_t line = 0;
     int pr = warp_probe_pin(d, page, line);
     if (pr == P_HIT) {
-      line_out = line;
       if (lane_id() == 0 && round == 0) atomicAdd(stat_ptr(d, S_HITS), 1ull);
-      return true;
+      return line;
     }
-    if (!(kCall ? warp_request_call(d, lane_id() == 0, page, q0, true, deadline)
-                : warp_request(d, lane_id() == 0, page, q0, true, deadline)))
-      return false;
-    if (aborted(d)) return false;
+    if (pr == P_BUSY) {
+      if (lane_id() == 0) {
+        if (round == 0) atomicAdd(stat_ptr(d, S_BUSY_HITS), 1ull);
+        for (uint32_t spin = 0;; ++spin) {
+          uint64_t t = ld_rlx64(&d.tag[line]);
+          if (tag_page(t) != page || tag_state(t) != ST_BUSY) break;
+          if ((spin & 7) == 7 && (gtimer() > deadline || aborted(d))) break;
+          __nanosleep(32);
+        }
+      }
+      __syncwarp();
+    } else if (!warp_request(d, lane_id() == 0, page, q0, false, deadline)) {
+      return kNoLine;
+    } else if (round) {
+      backoff(ns, 256);  // nothing could be evicted, or the page was evicted at once
+    }
+    if (aborted(d)) return kNoLine;
     if (gtimer() > deadline) {
       if (lane_id() == 0) set_error(d, -110);
-      return false;
+      return kNoLine;
     }
   }
+}
+static __device__ __forceinline__ bool warp_pin_page(const Dev &, uint64_t page, uint32_t q0, uint64_t deadline,
+                                                     uint32_t &line_out) {
+  line_out = warp_pin_page_body(page, q0, deadline);
+  return line_out != kNoLine;
 }
 
 // Asynchronous requests ahead of use pay a probe per page even when they have nothing
@@ -1056,10 +1257,9 @@ static __device__ uint64_t api_issue_read(const Dev &d, const AppCtx &a, bool wa
   bool need = leader;
   uint32_t ns = 64;
   while (__any_sync(kFull, need)) {
-    bool ring = false;
-    Issued is{};
     if (need) {
       uint32_t line = 0;
+      Issued is{};
       int pr = cache_probe(d, page, false, line);
       if (pr == P_HIT) {
         need = false;
@@ -1071,7 +1271,6 @@ static __device__ uint64_t api_issue_read(const Dev &d, const AppCtx &a, bool wa
         }
       } else {
         int m = cache_miss(d, page, a.q0, line, is);
-        ring = m == M_ISSUED;
         if (m == M_ISSUED) {
           tok = make_token(is.q, is.slot, is.ticket);
           need = false;
@@ -1081,7 +1280,6 @@ static __device__ uint64_t api_issue_read(const Dev &d, const AppCtx &a, bool wa
       }
       if (need && (gtimer() > a.deadline || aborted(d))) need = false;
     }
-    warp_ring(d, ring, is.q, is.slot, is.ticket, a.deadline);
     if (__any_sync(kFull, need)) backoff(ns, 1024);
   }
   tok = __shfl_sync(kFull, tok, lead & 31);
@@ -1110,7 +1308,7 @@ __device__ __forceinline__ int api_wait(const Dev &d, uint64_t tok, uint64_t dea
 // read completed is requested again.  False on a timeout of the launch.
 static __device__ bool api_copy_page(const Dev &d, const AppCtx &a, uint64_t page, void *dst) {
   uint32_t line;
-  if (!warp_pin_page<true>(d, page, a.q0, a.deadline, line)) return false;
+  if (!warp_pin_page(d, page, a.q0, a.deadline, line)) return false;
   warp_copy_page(dst, line_ptr(d, line));
   __syncwarp();
   if (lane_id() == 0) cache_unpin(d, line);
@@ -1128,7 +1326,7 @@ static __device__ bool api_get_row(const Dev &d, const AppCtx &a, uint64_t page,
     return false;
   }
   uint32_t line;
-  if (!warp_pin_page<true>(d, page, a.q0, a.deadline, line)) return false;
+  if (!warp_pin_page(d, page, a.q0, a.deadline, line)) return false;
   const uint8_t *src = line_ptr(d, line) + off;
   int32_t *o = (int32_t *)dst;
   for (uint32_t i = lane_id(); i < nbytes / 4; i += 32) o[i] = ld_cg_s32(src + 4 * i);
@@ -1179,54 +1377,76 @@ __device__ __forceinline__ void sum_rows(const Dev &d, uint32_t j0, uint32_t k, 
 }
 
 // Sum-pool rows begin..cnt-1 into acc, added in increasing lane order (lane j holds row
-// j's page `pg` and byte offset `off`).  Lane l adds the
-// float4 columns l, l+32, ... (MF4 of them, dim/4 in total).
-// Each round pins, in parallel, the distinct pages of the rows not yet added (one
-// probe per distinct page), adds the longest run of rows from the next one whose pages
-// are all pinned, and lets every pin go.  When the next row's page is not READY, the
-// warp requests all missing pages without waiting, then waits for and pins that one
-// page (nothing else pinned meanwhile, Sec. 2.3.2) and adds its row: every round adds
-// at least one row, whatever the set conflicts among the rows.
+// j's page `pg` and byte offset `off`).  Lane l adds the float4 columns l, l+32, ... (MF4
+// of them, dim/4 in total).
+// Each round probes the distinct pages of the rows not yet added, without pinning.  Of
+// those not READY, the first `window` ones that nobody has requested are requested
+// without waiting (the window keeps what all running warps have requested and not yet
+// used within the cache; rows that hit do not count, so that a bag of mostly resident
+// rows is one or two rounds).  Then the pages of the leading run of READY rows are
+// pinned, the run is added and every pin let go.  When the next row's page is not READY
+// the warp waits for and pins that one page (nothing else pinned meanwhile, Sec. 2.3.2)
+// and adds its row: every round adds at least one row, whatever the set conflicts.
 // `missed` (optional) is set in every lane when some page had to be requested.
 template <int MF4>
 static __device__ bool gather_sum(const Dev &d, const AppCtx &a, uint32_t begin, uint32_t cnt, uint64_t pg, uint32_t off,
-                           uint32_t nf4, float4 (&acc)[MF4], bool *missed = nullptr) {
+                           uint32_t nf4, float4 (&acc)[MF4], uint32_t window, bool *missed = nullptr) {
   unsigned l = lane_id();
   uint32_t j0 = begin;
   bool first = true;
+  const unsigned grp = __match_any_sync(kFull, l >= begin && l < cnt ? pg : ~0ull);
   while (j0 < cnt) {
     bool act = l >= j0 && l < cnt;
-    unsigned grp = __match_any_sync(kFull, act ? pg : ~0ull);
-    int lead_lane = __ffs(grp) - 1;
+    int lead_lane = __ffs(grp & (~0u << j0)) - 1;  // lowest lane of the page not yet added
     bool leader = act && lead_lane == (int)l;
     if (first) stat_warp(d, S_WARP_COALESCED, (act && !leader) ? 1u : 0u);
     uint32_t line = 0;
-    int pr = P_MISS;
-    if (leader) pr = cache_probe(d, pg, true, line);
+    int pr = P_HIT;
+    if (leader) pr = cache_probe(d, pg, false, line);
     if (first) stat_warp(d, S_HITS, (leader && pr == P_HIT) ? 1u : 0u);
     first = false;
-    bool lhit = __shfl_sync(kFull, (int)(pr == P_HIT), lead_lane & 31) != 0;
-    uint32_t myline = __shfl_sync(kFull, line, lead_lane & 31);
-    unsigned hm = __ballot_sync(kFull, act && lhit);
+    const unsigned away = __ballot_sync(kFull, leader && pr != P_HIT);
+    const bool ask = leader && pr == P_MISS && (uint32_t)__popc(away & ((1u << l) - 1)) < window;
+    // a request costs the warp the same few microseconds for one page as for many: the
+    // window is refilled when half of it has come in, or the next row needs it
+    const unsigned flying = __ballot_sync(kFull, leader && pr == P_BUSY);
+    const bool refill = 2 * (uint32_t)__popc(flying) < window || (away & -away & ~flying);
+    if (__any_sync(kFull, ask) && refill) {
+      if (missed) *missed = true;
+      if (!warp_request(d, ask, pg, a.q0, false, a.deadline)) return false;
+    }
+    // the leading run: its leaders pin
+    unsigned hm = __ballot_sync(kFull, act && !((away >> (lead_lane & 31)) & 1u));
     unsigned run = ~(hm >> j0);
     uint32_t k = run ? (uint32_t)(__ffs(run) - 1) : 32u;
     k = min(k, cnt - j0);
-    if (k) sum_rows<MF4>(d, j0, k, myline, off, nf4, acc);
-    __syncwarp();
-    if (leader && pr == P_HIT) cache_unpin(d, line);
     if (k) {
+      const bool mine = leader && l < j0 + k;
+      bool got = false;
+      if (mine) {
+        uint64_t old = atom_add_acq(&d.tag[line], PIN1);  // line data is read after the pin
+        uint64_t ost = tag_state(old);
+        got = tag_page(old) == pg && (ost == ST_READY || ost == ST_MODIFIED);
+        if (!got) cache_unpin(d, line);  // evicted since the probe
+      }
+      const unsigned lost = __ballot_sync(kFull, mine && !got);
+      uint32_t myline = __shfl_sync(kFull, line, lead_lane & 31);
+      if (lost) {
+        // rows of a lost page and those behind the first of them come in the next round
+        unsigned gone = __ballot_sync(kFull, act && ((lost >> (lead_lane & 31)) & 1u)) >> j0;
+        k = min(k, (uint32_t)(__ffs(gone) - 1));
+      }
+      if (k) sum_rows<MF4>(d, j0, k, myline, off, nf4, acc);
+      __syncwarp();
+      if (got) cache_unpin(d, line);
       j0 += k;
-      continue;
+      if (k) continue;
     }
-    // row j0's page is missing: request every missing page, then wait for row j0's
-    if (missed) *missed = true;
-    if (!warp_request(d, leader && pr != P_HIT, pg, a.q0, false, a.deadline)) return false;
+    // row j0's page is not READY: wait for it
     uint64_t pj = __shfl_sync(kFull, pg, j0 & 31);
     uint32_t lj;
     if (!warp_pin_page(d, pj, a.q0, a.deadline, lj)) return false;
-    uint32_t lines = __shfl_sync(kFull, myline, 0);  // placeholder value for other lanes
-    lines = (l == j0) ? lj : lines;
-    sum_rows<MF4>(d, j0, 1, lines, off, nf4, acc);
+    sum_rows<MF4>(d, j0, 1, lj, off, nf4, acc);
     __syncwarp();
     if (l == 0) cache_unpin(d, lj);
     j0 += 1;
@@ -1239,6 +1459,9 @@ static __device__ bool gather_sum(const Dev &d, const AppCtx &a, uint32_t begin,
 // Release what a completed command held (Sec. 3.2.1): the line becomes READY (or
 // INVALID on an error), the share-table entry is removed, the transaction barrier
 // (completion word) is set, the slot returns to EMPTY and the in-flight count drops.
+// The caller's fence after it read the completion entry orders the device's data before
+// the line's new state; one more fence orders everything before the slot and the
+// in-flight entry are free again.
 __device__ __forceinline__ void complete_command(const Dev &d, uint32_t q, uint32_t cid, uint32_t status) {
   uint64_t i = (uint64_t)q * d.depth + cid;
   uint64_t ctx = ld_rlx64(&d.cmd_ctx[i]);
@@ -1247,23 +1470,22 @@ __device__ __forceinline__ void complete_command(const Dev &d, uint32_t q, uint3
   uint64_t kind = ctx >> 60;
   uint32_t sh = (uint32_t)(ctx >> 32) & 0x0FFFFFFFu;
   uint32_t idx = (uint32_t)ctx;
-  fence_ar();
   if (kind == CTX_FILL) {
     if (status == 0) {
       atomicAdd(&d.tag[idx], 1ull);  // BUSY (1) -> READY (2)
     } else {
       atomicAnd(&d.tag[idx], PIN_MASK);  // back to INVALID
     }
-    sh_remove(d, sh);
   } else if (kind == CTX_WB) {
     if (idx) atomicAnd(&d.tag[idx - 1], ~TAG_WB);  // flush write-back from the line itself
-    sh_remove(d, sh);
-  } else if (kind == CTX_BUF) {
-    sh_remove(d, sh);
   }
+  const bool entry = kind == CTX_FILL || kind == CTX_WB || kind == CTX_BUF;
+  if (entry) st_rlx64(&d.sh_val[sh], 0ull);
   if (status) atomicAdd(stat_ptr(d, S_IO_ERRORS), 1ull);
-  st_rel64(&d.cmpl[i], ((ticket & 0xFFFFFFFFull) << 32) | ((uint64_t)(status & 0x7FFF) << 1) | 1ull);
-  st_rel64(&d.sqe_state[i], (ticket << 2) | SQE_EMPTY);
+  st_rlx64(&d.cmpl[i], ((ticket & 0xFFFFFFFFull) << 32) | ((uint64_t)(status & 0x7FFF) << 1) | 1ull);
+  fence_ar();
+  if (entry) sh_clear(d, sh);
+  st_rlx64(&d.sqe_state[i], (ticket << 2) | SQE_EMPTY);
   atomicAdd(&d.sq_resv[q], (unsigned long long)(-(int64_t)(1ull << 32)));
 }
 
@@ -1273,43 +1495,53 @@ __device__ __forceinline__ void complete_command(const Dev &d, uint32_t q, uint3
 // CQ doorbell.  The CQ has twice as many entries as the SQ, so with at most depth-1
 // commands outstanding and at most 31 consumed entries in the open window it never
 // fills (the device never has to wait for CQ space).
-static __device__ bool cq_poll(const Dev &d, uint32_t q) {
-  unsigned l = lane_id();
+// A dedicated poller keeps its position in registers (PollPos) for the whole launch.
+struct PollPos {
+  uint32_t offset, mask, phase;
+};
+__device__ __forceinline__ PollPos poll_load(const Dev &d, uint32_t q) {
+  const uint32_t *ps = &d.cq_poll[q * 4];
+  return PollPos{ld_rlx32(&ps[0]), ld_rlx32(&ps[1]), ld_rlx32(&ps[2])};
+}
+__device__ __forceinline__ void poll_store(const Dev &d, uint32_t q, const PollPos &p) {
   uint32_t *ps = &d.cq_poll[q * 4];
-  uint32_t offset = ld_rlx32(&ps[0]), mask = ld_rlx32(&ps[1]), phase = ld_rlx32(&ps[2]);
+  __syncwarp();
+  if (lane_id() == 0) {
+    st_rlx32(&ps[0], p.offset);
+    st_rlx32(&ps[1], p.mask);
+    st_rlx32(&ps[2], p.phase);
+  }
+  __syncwarp();
+}
+static __device__ bool cq_poll(const Dev &d, uint32_t q, PollPos &p) {
+  unsigned l = lane_id();
   uint32_t found = 0, windows = 0;
   for (int win = 0; win < 4; ++win) {
     bool valid = false;
-    if (!((mask >> l) & 1u)) {
-      Cqe *c = &d.cq[(uint64_t)q * d.cq_size + offset + l];
-      uint32_t w3 = ld_acq32(&c->dw[3]);
-      if (((w3 >> 16) & 1u) == phase) {
-        complete_command(d, q, w3 & 0xFFFFu, w3 >> 17);
-        valid = true;
-      }
+    uint32_t w3 = 0;
+    if (!((p.mask >> l) & 1u)) {
+      w3 = ld_rlx32(&d.cq[(uint64_t)q * d.cq_size + p.offset + l].dw[3]);
+      valid = ((w3 >> 16) & 1u) == p.phase;
     }
     unsigned b = __ballot_sync(kFull, valid);
+    if (!b) break;
+    fence_ar();  // an entry's phase was read: what the device wrote before it is visible now
+    if (valid) complete_command(d, q, w3 & 0xFFFFu, w3 >> 17);
     found += __popc(b);
-    mask |= b;
-    if (mask != kFull) break;
-    mask = 0;
-    offset += 32;
-    if (offset >= d.cq_size) {
-      offset = 0;
-      phase ^= 1u;
+    p.mask |= b;
+    if (p.mask != kFull) break;
+    p.mask = 0;
+    p.offset += 32;
+    if (p.offset >= d.cq_size) {
+      p.offset = 0;
+      p.phase ^= 1u;
     }
     ++windows;
     __syncwarp();
-    if (l == 0) {
-      fence_ar();
-      st_rel32(&d.cq_db[q], offset);
-    }
+    if (l == 0) st_rel32(&d.cq_db[q], p.offset);
   }
   __syncwarp();
   if (l == 0) {
-    st_rlx32(&ps[0], offset);
-    st_rlx32(&ps[1], mask);
-    st_rlx32(&ps[2], phase);
     if (found) atomicAdd(stat_ptr(d, S_CQES), (unsigned long long)found);
     if (windows) atomicAdd(stat_ptr(d, S_CQ_DOORBELLS), (unsigned long long)windows);
   }
@@ -1337,41 +1569,53 @@ constexpr uint32_t kEmuBatch = 2;
 constexpr uint64_t kEmuSlackNs = 16000;
 
 // Returns the number of commands served, or kEmuDevFull when commands were due but
-// their device was booked.  block_dev: a device this call may not book (a demand
-// command of the same engine pass is waiting for it), ~0u for none.
-constexpr uint32_t kEmuDevFull = 0x80000000u;
-static __device__ uint32_t emu_serve(const Dev &d, uint32_t q, uint32_t block_dev = ~0u) {
+// their device was booked, or kEmuLost when another engine took them.  f, db: the queue's fetch counter and doorbell as the caller's
+// scan has read them (uniform; db at least one command ahead).  block_dev: a device this
+// call may not book (a demand command of the same engine pass is waiting for it), ~0u
+// for none.
+constexpr uint32_t kEmuDevFull = 0x80000000u, kEmuLost = 0x40000000u;
+static __device__ uint32_t emu_serve(const Dev &d, uint32_t q, uint32_t f, uint32_t db, uint32_t block_dev = ~0u) {
   unsigned l = lane_id();
-  uint32_t *es = &d.emu[q * 4];
-  uint32_t f = 0, k = 0, full = 0;
+  uint32_t k = 0, full = 0;
   uint64_t now = gtimer();
   const uint32_t dv = d.ndev > 1 ? q % d.ndev : 0u;  // the device this queue belongs to
   const bool model = d.lat_ns || d.ns_per_page || d.ns_rd_dev || d.ns_wr_dev;
-  if (l == 0 && !model) {
-    // no latency model: every command the doorbell exposes is due at once.  The fetch
-    // counter is read before the doorbell, so with f still current (checked by the
-    // compare-and-swap) the doorbell is at most depth-1 commands ahead of it and
-    // (db - f) mod depth is the exact number of unfetched commands.
-    f = ld_acq32(&es[0]);
-    uint32_t db = ld_acq32(&d.sq_db[q]);
-    k = min((db - (f & d.dmask)) & d.dmask, kEmuBatch);
-    if (k && atomicCAS(&es[0], f, f + k) != f) k = 0;
+  fence_ar();  // the doorbell was read: the commands below it are visible now
+  __syncwarp();
+  int4 ea = make_int4(0, 0, 0, 0), eb = ea, ec = ea, eg = ea;
+  auto read_entry = [&]() {
+    if (l < k) {
+      const uint32_t *e = d.sq[(uint64_t)q * d.depth + ((f + l) & d.dmask)].dw;
+      ea = ld_cg16(e);
+      eb = ld_cg16(e + 4);
+      ec = ld_cg16(e + 8);
+      eg = ld_cg16(e + 12);
+    }
+  };
+  if (!model) {
+    // no latency model: every command the doorbell exposes is due at once.  Both counters
+    // only grow, so with f still current (checked by the compare-and-swap) the
+    // commands [f, db) are unfetched whichever of the two was read first.  The entries
+    // are read beside the compare-and-swap and used only if it succeeds.
+    k = min(db - f, kEmuBatch);
+    uint32_t got = f;
+    if (l == 0) got = atomicCAS(&d.emu_fetch[q], f, f + k);
+    read_entry();
+    got = __shfl_sync(kFull, got, 0);
+    if (got != f) return kEmuLost;
   } else if (l == 0) {
-    // `seen` must be read before the doorbell: it only ever takes doorbell values read
-    // earlier, so seen <= tail here and (db - seen) mod depth is the exact number of
-    // newly exposed commands (never a wrapped-around difference)
-    uint32_t seen = ld_acq32(&es[1]);
-    uint32_t db = ld_acq32(&d.sq_db[q]);
+    uint32_t seen = ld_acq32(&d.emu_seen[q]);
+    db = ld_acq32(&d.sq_db[q]);
     // stamp the arrival of commands the doorbell has newly exposed, then publish them
-    uint32_t fresh = (db - (seen & d.dmask)) & d.dmask;
-    if (fresh) {
+    uint32_t fresh = db - seen;
+    if ((int32_t)fresh > 0) {
       for (uint32_t i = 0; i < fresh; ++i)
         st_rlx64(&d.emu_arrival[(uint64_t)q * d.depth + ((seen + i) & d.dmask)], now);
       fence_ar();
-      atomicCAS(&es[1], seen, seen + fresh);
-      seen = ld_acq32(&es[1]);
+      atomicCAS(&d.emu_seen[q], seen, seen + fresh);
+      seen = ld_acq32(&d.emu_seen[q]);
     }
-    f = ld_rlx32(&es[0]);
+    f = ld_rlx32(&d.emu_fetch[q]);
     uint32_t avail = seen - f;
     if ((int32_t)avail > 0) {
       if (avail > kEmuBatch) avail = kEmuBatch;
@@ -1419,25 +1663,30 @@ static __device__ uint32_t emu_serve(const Dev &d, uint32_t q, uint32_t block_de
           if (!dbooked) k = 0;
         }
       }
-      if (k && atomicCAS(&es[0], f, f + k) != f) k = 0;
+      if (k && atomicCAS(&d.emu_fetch[q], f, f + k) != f) k = 0;
       if (!k) {
         if (qbooked) atomicAdd(&d.emu_busy[q], (unsigned long long)(-(int64_t)qcost));
         if (dbooked && dcost) atomicAdd(&d.dev_busy[dv], (unsigned long long)(-(int64_t)dcost));
       }
     }
   }
-  k = __shfl_sync(kFull, k, 0);
-  if (!k) return __shfl_sync(kFull, full, 0);
-  f = __shfl_sync(kFull, f, 0);
-  __syncwarp();  // lane 0's acquire of the doorbell orders the SQE reads of every lane
-  // command fields: lane i < k reads SQE f+i
+  if (model) {
+    k = __shfl_sync(kFull, k, 0);
+    if (!k) return __shfl_sync(kFull, full, 0);
+    f = __shfl_sync(kFull, f, 0);
+    __syncwarp();  // lane 0's acquire of the doorbell orders the reads of every lane
+    read_entry();
+  }
+  // the places of the completions, taken while the data moves (a completion queue holds
+  // every command in flight twice over)
+  uint32_t slot0 = 0;
+  if (l == 0) slot0 = atomicAdd(&d.emu_cqt[q], k);
+  // command fields: lane i < k holds those of SQE f+i
   uint32_t dw0 = 0, nlb = 0, status = 0;
   uint64_t prp1 = 0, slba = 0, t_commit = 0;
   bool drop = false;
   if (l < k) {
-    uint64_t i = (uint64_t)q * d.depth + ((f + l) & d.dmask);
-    const uint32_t *e = d.sq[i].dw;
-    int4 a = ld_cg16(e), b = ld_cg16(e + 4), c = ld_cg16(e + 8), g = ld_cg16(e + 12);
+    const int4 a = ea, b = eb, c = ec, g = eg;
     dw0 = (uint32_t)a.x;
     t_commit = (uint64_t)(uint32_t)a.z | ((uint64_t)(uint32_t)a.w << 32);
     prp1 = (uint64_t)(uint32_t)b.z | ((uint64_t)(uint32_t)b.w << 32);
@@ -1491,11 +1740,8 @@ static __device__ uint32_t emu_serve(const Dev &d, uint32_t q, uint32_t block_de
     if (opcode == OP_READ) atomicAdd(&d.pg_reads[slba], 1u);
     else if (opcode == OP_WRITE) atomicAdd(&d.pg_writes[slba], 1u);
   }
-  __threadfence();
   __syncwarp();
-  // completion entries
-  uint32_t slot0 = 0;
-  if (l == 0) slot0 = atomicAdd(&es[2], k);
+  // completion entries: the release of each orders the whole warp's data before it
   slot0 = __shfl_sync(kFull, slot0, 0);
   if (l < k) {
     uint32_t sl = slot0 + l;
@@ -1527,7 +1773,6 @@ static __device__ uint32_t emu_serve(const Dev &d, uint32_t q, uint32_t block_de
       st_rlx32(&c->dw[0], 0u);
       st_rlx32(&c->dw[1], 0u);
       st_rlx32(&c->dw[2], (q << 16) | ((f + l + 1) & d.dmask));
-      fence_ar();
       st_rel32(&c->dw[3], cid | (phase << 16) | (status << 17));
     }
   }
@@ -1541,23 +1786,43 @@ static __device__ uint32_t emu_serve(const Dev &d, uint32_t q, uint32_t block_de
 }
 
 // ================================================================ engine
-// One cooperative launch per library call.  Warp 0 of every CTA is a service warp:
-// an engine of the emulated device for every queue, and the Alg. 1 poller of queues
-// q = cta, cta + grid, ...  The other warps run the application.  No kernel of the
-// library ever waits on another launch: the device, the pollers and the waiters are
-// co-resident warps of one grid, and every wait is bounded by a deadline.
-// `sw` of `nsw`: this engine's number among the launch's engines (rotation start).
-static __device__ void service_loop(const Dev &d, uint32_t n_app, uint64_t deadline, bool poll, uint32_t sw,
-                                    uint32_t nsw) {
+// One cooperative launch per library call, one CTA per SM.  Of 19 CTAs three (evenly spread)
+// are service CTAs: their warps poll the completion queues (Alg. 1), one queue each where
+// there are enough of them, and are the engines of the emulated device for every queue.
+// The warps of the others run the application.  Service on SMs of its own, because the
+// miss path is bound by instruction supply as much as by L2 round trips: next to the
+// service loops a warp met 260 instruction-cache misses in a round of misses (ncu: 18 %
+// of an SM's fetches), and a computing warp slows the device down.
+// A launch of few CTAs has a service warp in each CTA instead, which does both.
+// No kernel of the library ever waits on another launch: the device, the pollers and the
+// waiters are co-resident warps of one grid, and every wait is bounded by a deadline.
+constexpr uint32_t kServiceNum = 3, kServiceDen = 19;  // 24 of 152 CTAs: 2,048 application warps are left
+struct Roles {
+  uint32_t svc;       // service CTAs (0: a service warp in every CTA)
+  uint32_t app_ctas;  // CTAs with application warps
+  uint32_t per_cta;   // application warps of each of them
+};
+__host__ __device__ __forceinline__ Roles engine_roles(uint32_t grid, uint32_t warps) {
+  Roles r;
+  r.svc = grid >= 8 ? grid * kServiceNum / kServiceDen : 0;
+  r.app_ctas = grid - r.svc;
+  r.per_cta = r.svc ? warps : warps - 1;
+  return r;
+}
+// `sw`: this engine's number (rotation start); the first `pollers` engines poll when `poll`.
+static __device__ void service_loop(const Dev &d, uint32_t app_ctas, uint64_t deadline, bool poll, uint32_t sw,
+                                    uint32_t pollers) {
   unsigned l = lane_id();
   uint32_t ns = 32;
   for (uint32_t iter = 0;; ++iter) {
-    bool progress = false;
-    // device engine: serve one queue per iteration, the first one with work found from
-    // a start that rotates over the queues and differs between engines, so that every
-    // queue is visited often and commands do not wait behind long scans
-    // (the doorbells and fetch counters of four windows of 32 queues are read in one
-    // round trip; they only select a queue, emu_serve checks them again)
+    bool progress = false, lost = false;
+    // device engine: serve one queue per iteration, one with work from a window of 32
+    // queues that rotates and differs between engines, so that every queue is visited
+    // often and commands do not wait behind long scans
+    // (the doorbells and fetch counters of a window are two 128-byte lines read in one
+    // round trip; they only select a queue, emu_serve checks them again.  Reading all
+    // 128 queues in every pass of every engine kept those few lines so busy that the
+    // threads' own doorbells and the compare-and-swaps on them queued up behind)
     // (demand queues first: the prefetch queues are served only when no demand queue
     // has a command the device may take now; a prefetch queue does not book a device
     // that a due demand command found booked in this pass, so the device's next free
@@ -1565,47 +1830,55 @@ static __device__ void service_loop(const Dev &d, uint32_t n_app, uint64_t deadl
     uint32_t block_dev = ~0u;
 #pragma unroll 1
     for (uint32_t cls = 0; cls < 2 && !progress; ++cls) {
-      uint32_t qsel = ~0u;
       const uint32_t base = cls ? d.Q - d.Qp : 0u, cnt = cls ? d.Qp : d.Q - d.Qp;
       if (cnt == 0) continue;
-      const uint32_t r = (uint32_t)(((uint64_t)iter * nsw + sw) % cnt);
       const uint32_t windows = (cnt + 31) / 32;
-      for (uint32_t w0 = 0; w0 < windows && qsel == ~0u; w0 += 4) {
-        uint32_t dbv[4], fv[4];
-#pragma unroll
-        for (uint32_t j = 0; j < 4; ++j) {
-          uint32_t off = (w0 + j) * 32 + l;
-          dbv[j] = fv[j] = 0;
-          if (off < cnt) {
-            uint32_t q = base + (r + off) % cnt;
-            dbv[j] = ld_rlx32(&d.sq_db[q]);
-            fv[j] = ld_rlx32(&d.emu[q * 4]);
-          }
+      // without prefetch queues any window will do; with them every demand queue is
+      // looked at before the first prefetch queue
+      const uint32_t looks = d.Qp ? windows : 1u;
+      uint32_t w = windows == 1 ? 0u : (iter + sw) % windows;
+      uint32_t qsel = ~0u, f = 0, db = 0;
+      for (uint32_t k = 0; k < looks && qsel == ~0u; ++k) {
+        const uint32_t off = w * 32 + l;
+        uint32_t dbv = 0, fv = 0;
+        if (off < cnt) {
+          dbv = ld_rlx32(&d.sq_db[base + off]);
+          fv = ld_rlx32(&d.emu_fetch[base + off]);
         }
-#pragma unroll
-        for (uint32_t j = 0; j < 4; ++j) {
-          uint32_t off = (w0 + j) * 32 + l;
-          unsigned m = __ballot_sync(kFull, off < cnt && ((dbv[j] - (fv[j] & d.dmask)) & d.dmask) != 0);
-          if (m && qsel == ~0u) qsel = base + (r + (w0 + j) * 32 + (uint32_t)(__ffs(m) - 1)) % cnt;
+        unsigned m = __ballot_sync(kFull, (int32_t)(dbv - fv) > 0);
+        if (m) {
+          const uint32_t turn = ((sw * 31 + iter) * 0x9E3779B1u) >> 27;  // engines start at different queues
+          const int at = (__ffs(__funnelshift_r(m, m, turn)) - 1 + turn) & 31;
+          qsel = base + w * 32 + at;
+          f = __shfl_sync(kFull, fv, at);
+          db = __shfl_sync(kFull, dbv, at);
         }
+        if (++w == windows) w = 0;
       }
       if (qsel != ~0u) {
-        uint32_t r = emu_serve(d, qsel, block_dev);
+        uint32_t r = emu_serve(d, qsel, f, db, block_dev);
         if (r == kEmuDevFull) block_dev = d.ndev > 1 ? qsel % d.ndev : 0u;
+        else if (r == kEmuLost) lost = true;
         else if (r) progress = true;
       }
     }
     // completion side (Alg. 1) for the queues this warp polls
     if (poll)
-      for (uint32_t q = sw; q < d.Q; q += nsw) progress |= cq_poll(d, q);
-    if (progress) {
+      for (uint32_t q = sw; q < d.Q; q += pollers) {
+        PollPos p = poll_load(d, q);
+        if (cq_poll(d, q, p)) {
+          poll_store(d, q, p);
+          progress = true;
+        }
+      }
+    if (progress || (lost && (iter & 7) != 7)) {  // another engine was faster: there is work, look again at once
       ns = 32;
       continue;
     }
     uint32_t done = 0;
     if (l == 0) done = ld_acq32(&d.run->app_done);
     done = __shfl_sync(kFull, done, 0);
-    if (done >= n_app) {
+    if (done >= app_ctas) {
       bool drained = true;
       for (uint32_t q = l; q < d.Q; q += 32)
         if ((ld_acq64(&d.sq_resv[q]) >> 32) != 0) drained = false;
@@ -1620,57 +1893,91 @@ static __device__ void service_loop(const Dev &d, uint32_t n_app, uint64_t deadl
   }
 }
 
-// A dedicated Alg. 1 poller of queue q: an application warp that sits out the call.
-// Ends when every application warp is done and the queue has nothing in flight.
-static __device__ void poller_loop(const Dev &d, uint32_t q, uint32_t n_app, uint64_t deadline) {
+// A dedicated Alg. 1 poller of the queues q, q + step, ...  Ends when every application
+// warp is done and its queues have nothing in flight.
+static __device__ void poller_loop(const Dev &d, uint32_t q0, uint32_t step, uint32_t app_ctas, uint64_t deadline) {
   unsigned l = lane_id();
-  uint32_t ns = 32;
-  for (;;) {
-    if (cq_poll(d, q)) {
-      ns = 32;
+  const bool one = q0 + step >= d.Q;
+  PollPos p = poll_load(d, q0);
+  for (uint32_t iter = 1;; ++iter) {
+    bool found = false;
+    if (one) {
+      found = cq_poll(d, q0, p);
+    } else {
+      for (uint32_t q = q0; q < d.Q; q += step) {
+        p = poll_load(d, q);
+        if (cq_poll(d, q, p)) {
+          poll_store(d, q, p);
+          found = true;
+        }
+      }
+    }
+    if (found) continue;
+    if (iter & 3) {  // the end of the call is looked for now and then
+      __nanosleep(32);
       continue;
     }
     uint32_t done = 0;
-    uint64_t resv = 0;
-    if (l == 0) {
-      done = ld_acq32(&d.run->app_done);
-      resv = ld_acq64(&d.sq_resv[q]);
-    }
+    if (l == 0) done = ld_acq32(&d.run->app_done);
     done = __shfl_sync(kFull, done, 0);
-    resv = __shfl_sync(kFull, resv, 0);
-    if (done >= n_app && (resv >> 32) == 0) break;
+    if (done >= app_ctas) {
+      bool drained = true;
+      for (uint64_t q = q0 + (uint64_t)l * step; q < d.Q; q += 32ull * step)
+        if ((ld_acq64(&d.sq_resv[q]) >> 32) != 0) drained = false;
+      if (__all_sync(kFull, drained)) break;
+    }
     if (gtimer() > deadline) {
       if (l == 0) set_error(d, -110);
       break;
     }
-    __nanosleep(ns);
-    ns = ns < 256 ? ns * 2 : 256;
   }
+  if (one) poll_store(d, q0, p);
 }
 
-// Grid barrier over the application warps only (service warps never join).
+// Grid barrier over the application warps only (service warps never join).  The warps of a
+// CTA meet in shared memory; the last one of each meets the others' in device memory (a
+// single counter for all 2,000 warps took 5 us of serialised atomics).
 static __device__ bool app_barrier(const Dev &d, uint32_t n_app, uint64_t deadline) {
+  (void)n_app;
+  CtaState &cs = cta_state();
   bool ok = true;
   __syncwarp();
   if (lane_id() == 0) {
+    volatile uint32_t *cgen = &cs.bar_gen;
+    const uint32_t mine = *cgen;
     fence_ar();
-    uint32_t gen = ld_acq32(&d.run->bar_gen);
-    uint32_t arrived = atomicAdd(&d.run->bar_count, 1u) + 1;
-    if (arrived == n_app) {
-      st_rlx32(&d.run->bar_count, 0u);
+    if (atomicAdd(&cs.bar_count, 1u) + 1 == cs.active) {
+      cs.bar_count = 0;
       fence_ar();
-      st_rel32(&d.run->bar_gen, gen + 1);
+      uint32_t gen = ld_acq32(&d.run->bar_gen);
+      if (atomicAdd(&d.run->bar_count, 1u) + 1 == cs.ctas_active) {
+        st_rlx32(&d.run->bar_count, 0u);
+        fence_ar();
+        st_rel32(&d.run->bar_gen, gen + 1);
+      } else {
+        uint32_t spin = 0;
+        while (ld_acq32(&d.run->bar_gen) == gen) {
+          if ((++spin & 15) == 0 && gtimer() > deadline) {
+            set_error(d, -110);
+            ok = false;
+            break;
+          }
+          __nanosleep(64);
+        }
+      }
+      fence_ar();
+      if (ok) *cgen = mine + 1;
     } else {
-      uint32_t ns = 32;
-      while (ld_acq32(&d.run->bar_gen) == gen) {
-        if (gtimer() > deadline) {
+      uint32_t spin = 0;
+      while (*cgen == mine) {
+        if ((++spin & 15) == 0 && gtimer() > deadline) {
           set_error(d, -110);
           ok = false;
           break;
         }
-        __nanosleep(ns);
-        ns = ns < 1024 ? ns * 2 : 1024;
+        __nanosleep(64);
       }
+      fence_ar();
     }
   }
   ok = __shfl_sync(kFull, ok, 0);
@@ -1679,8 +1986,8 @@ static __device__ bool app_barrier(const Dev &d, uint32_t n_app, uint64_t deadli
 }
 
 
-// CTAs per SM the engine is compiled for (register budget): App::kMinBlocks if the
-// application asks for more occupancy, else 2
+// Occupancy the engine is compiled for, in groups of kWarps warps per SM (register
+// budget): App::kMinBlocks if the application asks for more, else 2
 template <class App, class = void>
 struct MinBlocks {
   static constexpr int value = 2;
@@ -1689,50 +1996,89 @@ template <class App>
 struct MinBlocks<App, decltype((void)App::kMinBlocks, void())> {
   static constexpr int value = App::kMinBlocks;
 };
+template <class App>
+struct EngineShape {
+  static constexpr int warps = kWarps * MinBlocks<App>::value;
+  static constexpr int threads = warps * 32;
+};
+// dynamic shared memory an application wants for each warp of the CTA
+template <class App, class = void>
+struct SharedPerWarp {
+  static constexpr int value = 0;
+};
+template <class App>
+struct SharedPerWarp<App, decltype((void)App::kSharedPerWarp, void())> {
+  static constexpr int value = App::kSharedPerWarp;
+};
+template <class App>
+constexpr int engine_shared() {
+  return SharedPerWarp<App>::value * EngineShape<App>::warps;
+}
 
 template <class App>
-__global__ void __launch_bounds__(kThreads, MinBlocks<App>::value) engine_kernel(Dev d, App app) {
+__global__ void __launch_bounds__(EngineShape<App>::threads, 1)
+    engine_kernel(const __grid_constant__ Dev d, const __grid_constant__ App app) {
+  constexpr uint32_t kCtaWarps = EngineShape<App>::warps;
+  const Roles r = engine_roles(gridDim.x, kCtaWarps);
+  // service CTAs are evenly spread over the grid
+  const uint32_t before = (uint32_t)((uint64_t)blockIdx.x * r.svc / gridDim.x);
+  const bool svc_cta = (uint32_t)(((uint64_t)blockIdx.x + 1) * r.svc / gridDim.x) != before;
+  const uint32_t app_cta = blockIdx.x - before;
+  const uint32_t n_app = r.app_ctas * r.per_cta;
+  const uint32_t n_active = (d.app_active && d.app_active < n_app) ? d.app_active : n_app;
+  CtaState &cs = cta_state();
+  static_assert(sizeof(Dev) % 4 == 0, "copied in 4-byte words");
+  for (uint32_t i = threadIdx.x; i < sizeof(Dev) / 4; i += EngineShape<App>::threads)
+    ((uint32_t *)&cs.dev)[i] = ((const uint32_t *)&d)[i];
+  if (threadIdx.x == 0) {
+    cs.done = cs.bar_count = cs.bar_gen = 0;
+    cs.active = n_active > app_cta ? (n_active - app_cta + r.app_ctas - 1) / r.app_ctas : 0;
+    cs.ctas_active = n_active < r.app_ctas ? n_active : r.app_ctas;
+  }
+  __syncthreads();
   uint32_t warp = threadIdx.x >> 5;
-  uint32_t n_app = gridDim.x * (kWarps - 1);
   uint64_t deadline = gtimer() + (d.session_ns ? d.session_ns : d.timeout_ns);
-  uint32_t n_active = (d.app_active && d.app_active < n_app) ? d.app_active : n_app;
-  // when at least Q application warps sit out the call, the first Q of them poll one
-  // queue each, and the service warps only serve the device
-  const bool pollers = n_app - n_active >= d.Q;
-  if (warp == 0) {
-    uint32_t idle = n_app - n_active, q_used = pollers ? d.Q : 0;
-    uint32_t extra = idle > q_used ? min(idle - q_used, d.extra_engines) : 0;
-    service_loop(d, n_app, deadline + d.timeout_ns, !pollers, blockIdx.x, gridDim.x + extra);
-    return;
-  }
   AppCtx a;
-  a.warp = blockIdx.x * (kWarps - 1) + (warp - 1);
+  // consecutive application warps are on different CTAs: a call that runs a few hundred
+  // warps has them on as many SMs, and they seldom wait for each other's issue slots
+  const uint32_t first_app = kCtaWarps - r.per_cta;
+  a.warp = (warp - first_app) * r.app_ctas + app_cta;
   a.n_warps = n_active;
-  if (a.warp >= a.n_warps) {
-    // not needed by this call: keeps the working set of the active warps in the cache.
-    // The first Q such warps poll a completion queue each (when there are Q of them),
-    // the next ones (up to d.extra_engines) serve the device as additional engines.
-    if (lane_id() == 0) atomicAdd(&d.run->app_done, 1u);
-    uint32_t idle = a.warp - a.n_warps, q_used = pollers ? d.Q : 0;
-    if (idle < q_used) {
-      poller_loop(d, idle, n_app, deadline + d.timeout_ns);
-    } else {
-      uint32_t extra = min(n_app - n_active - q_used, d.extra_engines);
-      if (idle - q_used < extra)
-        service_loop(d, n_app, deadline + d.timeout_ns, false, gridDim.x + (idle - q_used), gridDim.x + extra);
+  bool serve = true, poll = false;
+  uint32_t sw = blockIdx.x;
+  if (svc_cta) {
+    const uint32_t n_svc = r.svc * kCtaWarps, me = warp * r.svc + before;
+    const uint32_t n_poll = min(d.Q, n_svc / 3);
+    if (me < n_poll) {
+      poller_loop(d, me, n_poll, r.app_ctas, deadline + d.timeout_ns);
+      return;
     }
-    return;
+    sw = me - n_poll;
+  } else if (warp < first_app) {
+    poll = true;
+  } else {
+    // application warps beyond n_active are not needed by this call (the working set of the
+    // active ones stays in the cache)
+    if (a.warp < n_active) {
+      // home queue by thread index, spread so that the lanes of a warp and the lane 0 of
+      // consecutive warps all start on different queues
+      a.q0 = (uint32_t)((a.warp + (uint64_t)lane_id() * ((d.Q + 31) / 32)) % d.Q);
+      a.deadline = deadline;
+      app.run(d, a);
+      __syncwarp();
+    }
+    if (lane_id() == 0) {
+      fence_ar();
+      if (atomicAdd(&cs.done, 1u) + 1 == r.per_cta) {
+        fence_ar();
+        atomicAdd(&d.run->app_done, 1u);
+      }
+    }
+    serve = a.warp >= n_active && a.warp - n_active < d.extra_engines;
+    sw = gridDim.x + a.warp;
   }
-  // home queue by thread index, spread so that the lanes of a warp and the lane 0 of
-  // consecutive warps all start on different queues
-  a.q0 = (uint32_t)((a.warp + (uint64_t)lane_id() * ((d.Q + 31) / 32)) % d.Q);
-  a.deadline = deadline;
-  app.run(d, a);
-  __syncwarp();
-  if (lane_id() == 0) {
-    fence_ar();
-    atomicAdd(&d.run->app_done, 1u);
-  }
+  // (one call site: the engines of an SM share its instruction cache)
+  if (serve) service_loop(d, r.app_ctas, deadline + d.timeout_ns, poll, sw, gridDim.x);
 }
 
 }  // namespace agile

@@ -144,7 +144,6 @@ struct WriteApp {
         backoff(ns);
       }
       line = __shfl_sync(kFull, line, 0);
-      if (!warp_ring(d, l == 0 && is.q != 0xFFFFFFFFu, is.q, is.slot, is.ticket, a.deadline)) return;
       // 3. new contents into the line; publish it READY (a full page supersedes it)
       warp_copy_page(line_ptr(d, line), src + i * kPage);
       __threadfence();
@@ -185,11 +184,11 @@ struct WriteApp {
         __threadfence();
         __syncwarp();
         if (l == 0) {
-          sq_commit(d, q, slot, ticket, OP_WRITE, (uint64_t)stg, page, ctx_make(CTX_WB, (uint32_t)sh, 0));
+          sq_write(d, q, slot, ticket, OP_WRITE, (uint64_t)stg, page, ctx_make(CTX_WB, (uint32_t)sh, 0));
           atomicAdd(stat_ptr(d, S_WRITEBACKS), 1ull);
           cache_unpin(d, line);
+          sq_ring(d, q, ticket);
         }
-        if (!warp_ring(d, l == 0, q, slot, ticket, a.deadline)) return;
         t = make_token(q, slot, ticket);
       } else if (l == 0) {
         // no queue slot: keep the data as a MODIFIED line, written back later
@@ -254,11 +253,11 @@ struct FlushApp {
         __syncwarp();
         if (mine) {
           uint8_t *stg = d.staging + ((uint64_t)q * d.depth + slot) * kPage;
-          sq_commit(d, q, slot, ticket, OP_WRITE, (uint64_t)stg, tag_page(t),
-                    ctx_make(CTX_WB, (uint32_t)sh, (uint32_t)(line + 1)));
+          sq_write(d, q, slot, ticket, OP_WRITE, (uint64_t)stg, tag_page(t),
+                   ctx_make(CTX_WB, (uint32_t)sh, (uint32_t)(line + 1)));
           atomicAdd(stat_ptr(d, S_WRITEBACKS), 1ull);
+          sq_ring(d, q, ticket);
         }
-        if (!warp_ring(d, mine, q, slot, ticket, a.deadline)) return;
       }
       if (!__any_sync(kFull, dirty_left)) return;
       if (gtimer() > a.deadline || aborted(d)) {
@@ -287,7 +286,7 @@ struct ReplayApp {
       }
       uint32_t ns = 64;
       for (;;) {
-        int done = 0, issued = 0, ring = 0;
+        int done = 0, issued = 0;
         uint32_t line = 0;
         Issued is{};
         if (l == 0) {
@@ -297,7 +296,6 @@ struct ReplayApp {
             atomicAdd(stat_ptr(d, S_HITS), 1ull);
           } else if (pr == P_MISS) {
             int m = cache_miss(d, page, a.q0, line, is);
-            ring = m == M_ISSUED;
             if (m == M_ISSUED) {
               issued = 1;
               code = is.code;
@@ -307,7 +305,6 @@ struct ReplayApp {
         done = __shfl_sync(kFull, done, 0);
         if (done) break;
         issued = __shfl_sync(kFull, issued, 0);
-        if (!warp_ring(d, l == 0 && ring, is.q, is.slot, is.ticket, a.deadline)) return;
         if (issued) {
           // wait for the fill with nothing held
           line = __shfl_sync(kFull, line, 0);
@@ -495,7 +492,12 @@ int agile_init(const agile_config *cfg_in, agile_ctx **out) {
   uint64_t Q = cfg.num_queues, D = dep;
   uint32_t buckets = 1024;
   while ((uint64_t)buckets < Q * D) buckets <<= 1;
-  d.sh_mask = buckets - 1;
+  // four 16-bit slots a bucket (15 bits tell the pages of a bucket apart): enough buckets
+  // for every command in flight and for every page number of the store
+  while (((uint64_t)buckets << kShKeyBits) < cfg.store_bytes / kPage) buckets <<= 1;
+  d.sh_bits = kShKeyBits;
+  while ((1u << (d.sh_bits - kShKeyBits)) < buckets) d.sh_bits++;
+  d.sh_mul = (0x9E3779B97F4A7C15ull >> (64 - d.sh_bits)) | 1ull;
   d.Q = (uint32_t)Q;
   d.Qp = (uint32_t)prefetch_queue_count(cfg.prefetch_queues, cfg.num_queues, cfg.num_devices);
   d.depth = dep;
@@ -512,7 +514,7 @@ int agile_init(const agile_config *cfg_in, agile_ctx **out) {
   d.lines = (uint8_t *)A(d.nlines * kPage);
   d.tag = (unsigned long long *)A(d.nlines * 8);
   d.hand = (uint32_t *)A(sets * 4);
-  d.sh_key = (unsigned long long *)A((uint64_t)buckets * 4 * 8);
+  d.sh_key = (unsigned long long *)A((uint64_t)buckets * 8);
   d.sh_val = (unsigned long long *)A((uint64_t)buckets * 4 * 8);
   d.sq = (Sqe *)A(Q * D * sizeof(Sqe));
   d.cq_size = 2 * dep;
@@ -521,12 +523,12 @@ int agile_init(const agile_config *cfg_in, agile_ctx **out) {
   d.cmd_ctx = (unsigned long long *)A(Q * D * 8);
   d.cmpl = (unsigned long long *)A(Q * D * 8);
   d.sq_resv = (unsigned long long *)A(Q * 8);
-  d.sq_tail = (uint32_t *)A(Q * 4);
-  d.sq_lock = (uint32_t *)A(Q * 4);
   d.sq_db = (uint32_t *)A(Q * 4);
   d.cq_db = (uint32_t *)A(Q * 4);
   d.cq_poll = (uint32_t *)A(Q * 16);
-  d.emu = (uint32_t *)A(Q * 16);
+  d.emu_fetch = (uint32_t *)A(Q * 4);
+  d.emu_seen = (uint32_t *)A(Q * 4);
+  d.emu_cqt = (uint32_t *)A(Q * 4);
   d.emu_busy = (unsigned long long *)A(Q * 8);
   d.emu_arrival = (unsigned long long *)A(Q * D * 8);
   d.staging = (uint8_t *)A(Q * D * kPage);
@@ -577,7 +579,7 @@ int agile_init(const agile_config *cfg_in, agile_ctx **out) {
   d.timeout_ns = cfg.wait_timeout_ns;
   d.extra_engines = cfg.emu_extra_engines == AGILE_NO_EXTRA_ENGINES
                         ? 0u
-                        : (cfg.emu_extra_engines ? cfg.emu_extra_engines : 0xFFFFFFFFu);
+                        : cfg.emu_extra_engines;
   d.prefetch_depth = cfg.prefetch_depth;
   if (cudaDeviceSynchronize() != cudaSuccess) {
     agile_destroy(c);
@@ -760,12 +762,7 @@ int agile_set_device_model(agile_ctx *c, uint32_t ndev, uint32_t lat_ns, double 
   // The device without a model advances only its fetch counters; with a model it also
   // counts the commands it has seen (arrival stamps).  Between calls every command has
   // been served, so each queue's "seen" counter is set to its fetch counter.
-  {
-    std::vector<uint32_t> emu((size_t)c->dev.Q * 4);
-    AGILE_CUDA_TRY(cudaMemcpy(emu.data(), c->dev.emu, emu.size() * 4, cudaMemcpyDeviceToHost));
-    for (uint64_t q = 0; q < c->dev.Q; ++q) emu[q * 4 + 1] = emu[q * 4];
-    AGILE_CUDA_TRY(cudaMemcpy(c->dev.emu, emu.data(), emu.size() * 4, cudaMemcpyHostToDevice));
-  }
+  AGILE_CUDA_TRY(cudaMemcpy(c->dev.emu_seen, c->dev.emu_fetch, (size_t)c->dev.Q * 4, cudaMemcpyDeviceToDevice));
   c->cfg.num_devices = std::max(c->cfg.num_devices, ndev);
   c->dev.ndev = ndev;
   c->dev.Qp = (uint32_t)qp;
@@ -874,7 +871,7 @@ int agile_config_parallelism(agile_ctx *c, uint32_t app_warps) {
 int agile_launch_shape(agile_ctx *c, uint32_t *ctas, uint32_t *threads) {
   if (!c) return AGILE_EINVAL;
   if (ctas) *ctas = (uint32_t)engine_grid<ReadApp>(c);
-  if (threads) *threads = kThreads;
+  if (threads) *threads = EngineShape<ReadApp>::threads;
   return AGILE_OK;
 }
 

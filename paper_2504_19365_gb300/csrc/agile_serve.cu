@@ -160,10 +160,7 @@ struct ServeApp {
       uint64_t byte = r * dim * 4;
       if (mode == AGILE_ASYNC && !warp_request(d, l < cnt, page0 + byte / kPage, a.q0, false, a.deadline))
         return false;
-      for (uint32_t g0 = 0; g0 < cnt; g0 += group) {
-        uint32_t g1 = min(cnt, g0 + group);
-        if (!gather_sum<1>(d, a, g0, g1, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc)) return false;
-      }
+      if (!gather_sum<1>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, group)) return false;
     }
     if (l < nf4) ((float4 *)(out + (uint64_t)b * dim))[l] = acc[0];
     return true;

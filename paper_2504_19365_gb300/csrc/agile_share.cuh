@@ -103,10 +103,9 @@ static __device__ __forceinline__ void ub_ready(const Dev &d, uint64_t k, uint64
   }
 }
 
-// One attempt to fill the new entry k of `page` into `mine`: 1 done (*tok set; *ring
-// when a read command was committed to `is`), 0 try again later.
-static __device__ int ub_fill(const Dev &d, const AppCtx &a, uint64_t page, uint8_t *mine, uint64_t k, uint64_t &tok,
-                       Issued &is, bool &ring) {
+// One attempt to fill the new entry k of `page` into `mine`: 1 done (*tok set; a read may
+// have been issued), 0 try again later.
+static __device__ int ub_fill(const Dev &d, const AppCtx &a, uint64_t page, uint8_t *mine, uint64_t k, uint64_t &tok) {
   int64_t sh = sh_insert(d, page, SH_FILL);
   if (sh < 0) return 0;  // the page is in flight (a fill or a write-back): later
   uint32_t line = 0;
@@ -129,28 +128,24 @@ static __device__ int ub_fill(const Dev &d, const AppCtx &a, uint64_t page, uint
     sh_remove(d, (uint64_t)sh);
     return 0;
   }
-  sq_commit(d, q, slot, ticket, OP_READ, (uint64_t)mine, page, ctx_make(CTX_BUF, (uint32_t)sh, 0));
+  sq_write(d, q, slot, ticket, OP_READ, (uint64_t)mine, page, ctx_make(CTX_BUF, (uint32_t)sh, 0));
   atomicAdd(stat_ptr(d, S_MISSES), 1ull);
+  sq_ring(d, q, ticket);
   tok = make_token(q, slot, ticket);
-  is.q = q;
-  is.slot = slot;
-  is.ticket = ticket;
-  ring = true;
   ub_ready(d, k, tok);
   return 1;
 }
 
 // One attempt to write the buffer of a closing modified entry into the page's cache
 // line: 1 done, 0 try again later.  `sh` keeps the page's in-flight entry across
-// attempts (-1: not taken yet); a write-back of the line's victim may be committed to
-// `is` (*ring).
-static __device__ int ub_propagate(const Dev &d, const AppCtx &a, uint64_t page, const uint8_t *buf, int64_t &sh, Issued &is,
-                            bool &ring) {
+// attempts (-1: not taken yet); a write-back of the line's victim may be issued.
+static __device__ int ub_propagate(const Dev &d, const AppCtx &a, uint64_t page, const uint8_t *buf, int64_t &sh) {
   if (sh < 0) {
     sh = sh_insert(d, page, SH_WRITE);
     if (sh < 0) return 0;
   }
   uint32_t line = 0;
+  Issued is{};
   int pr = cache_probe(d, page, true, line);
   if (pr == P_HIT) {
     lane_copy_page(line_ptr(d, line), buf);
@@ -165,7 +160,6 @@ static __device__ int ub_propagate(const Dev &d, const AppCtx &a, uint64_t page,
   if (pr == P_BUSY) return 0;
   int m = cache_miss(d, page, a.q0, line, is, false, sh);
   if (m != M_ISSUED) return 0;
-  ring = is.q != 0xFFFFFFFFu;  // a MODIFIED victim's write-back
   lane_copy_page(line_ptr(d, line), buf);
   fence_ar();
   atomicAdd(&d.tag[line], 2ull);  // BUSY (1) -> MODIFIED (3)
@@ -190,9 +184,6 @@ static __device__ int share_acquire(const Dev &d, const AppCtx &a, bool want, ui
   uint64_t tok = ~0ull;
   uint32_t ns = 64;
   while (__any_sync(kFull, phase < 3)) {
-    bool ring = false;
-    Issued is{};
-    is.q = 0xFFFFFFFFu;
     bool moved = false;
     if (phase == 0) {
       k = ub_find(d, page);
@@ -213,7 +204,7 @@ static __device__ int share_acquire(const Dev &d, const AppCtx &a, bool want, ui
       }
     }
     if (phase == 1) {
-      if (ub_fill(d, a, page, mine, (uint64_t)k, tok, is, ring)) {
+      if (ub_fill(d, a, page, mine, (uint64_t)k, tok)) {
         phase = 3;
         moved = true;
       }
@@ -225,7 +216,6 @@ static __device__ int share_acquire(const Dev &d, const AppCtx &a, bool want, ui
         phase = 3;
       }
     }
-    warp_ring(d, ring, is.q, is.slot, is.ticket, a.deadline);
     if (phase < 3 && !moved && gtimer() > a.deadline) {
       rc = AGILE_ETIMEDOUT;  // an entry set up by this lane stays PENDING: the launch is failing anyway
       set_error(d, -110);
@@ -267,9 +257,6 @@ static __device__ int share_release(const Dev &d, const AppCtx &a, bool want, ui
   const uint8_t *buf = nullptr;
   uint32_t ns = 64;
   while (__any_sync(kFull, phase < 2)) {
-    bool ring = false;
-    Issued is{};
-    is.q = 0xFFFFFFFFu;
     bool moved = false;
     if (phase == 0) {
       k = ub_find(d, page);
@@ -293,7 +280,7 @@ static __device__ int share_release(const Dev &d, const AppCtx &a, bool want, ui
         }
       }
     }
-    if (phase == 1 && ub_propagate(d, a, page, buf, sh, is, ring)) {
+    if (phase == 1 && ub_propagate(d, a, page, buf, sh)) {
       rc = 1;
       phase = 3;
       moved = true;
@@ -305,7 +292,6 @@ static __device__ int share_release(const Dev &d, const AppCtx &a, bool want, ui
       st_rel64(&d.ub_key[k], 0ull);
       phase = 2;
     }
-    warp_ring(d, ring, is.q, is.slot, is.ticket, a.deadline);
     if (phase < 2 && !moved && gtimer() > a.deadline) {
       rc = AGILE_ETIMEDOUT;
       set_error(d, -110);
