@@ -93,13 +93,15 @@ static __device__ unsigned long long g_launch_seq;
 
 // Zero the per-launch state and give the launch its number (RunState::epoch).  Runs on
 // the call's stream right before the engine kernel.
-static __global__ void run_reset_kernel(RunState *r) {
+// (by one CTA)
+static __device__ __forceinline__ void run_reset(RunState *r) {
   static_assert(sizeof(RunState) % 4 == 0, "RunState is cleared in 4-byte words");
   uint32_t *w = (uint32_t *)r;
   for (uint32_t i = threadIdx.x; i < sizeof(RunState) / 4; i += blockDim.x) w[i] = 0u;
   __syncthreads();
   if (threadIdx.x == 0) r->epoch = atomicAdd(&g_launch_seq, 1ull) + 1ull;
 }
+static __global__ void run_reset_kernel(RunState *r) { run_reset(r); }
 
 // `active`: application warps the call wants (0 = every app warp of the grid); the
 // context's app_warps setting overrides it.
@@ -111,14 +113,17 @@ struct has_demand_only : std::false_type {};
 template <class T>
 struct has_demand_only<T, std::void_t<decltype(std::declval<const T &>().demand_only())>> : std::true_type {};
 
+// `reset`: false when a kernel launched right before has already reset the run state.
 template <class App>
-int launch_engine(agile_ctx *c, const App &app, void *stream, uint32_t active = 0) {
+int launch_engine(agile_ctx *c, const App &app, void *stream, uint32_t active = 0, bool reset = true) {
   cudaStream_t s = as_stream(stream);
   AGILE_CUDA_TRY(cudaSetDevice(c->device));
   int grid = engine_grid<App>(c);
   if (grid <= 0) return AGILE_ECUDA;
-  run_reset_kernel<<<1, 128, 0, s>>>(c->dev.run);
-  AGILE_CUDA_TRY(cudaGetLastError());
+  if (reset) {
+    run_reset_kernel<<<1, 128, 0, s>>>(c->dev.run);
+    AGILE_CUDA_TRY(cudaGetLastError());
+  }
   Dev d = c->dev;
   d.app_active = c->cfg.app_warps ? c->cfg.app_warps : active;
   if constexpr (has_demand_only<App>::value) {

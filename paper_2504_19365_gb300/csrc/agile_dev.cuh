@@ -76,6 +76,8 @@ struct RunState {
   uint32_t work[4];       // dynamic work counters
   unsigned long long acc[4];  // accumulators (edges scanned, discovered vertices, ...)
   uint32_t flag[4];
+  uint32_t pending;       // bags the resident pass of a lookup has left to the engine
+  uint32_t pad;
   unsigned long long epoch;  // number of this launch among the device's launches (never 0)
   // BFS slice queue, per level parity, each on a line of its own (hot words)
   alignas(128) uint32_t hub_count[2];  // slices of long adjacency lists reserved
@@ -1813,12 +1815,12 @@ __host__ __device__ __forceinline__ Roles engine_roles(uint32_t grid, uint32_t w
 static __device__ void service_loop(const Dev &d, uint32_t app_ctas, uint64_t deadline, bool poll, uint32_t sw,
                                     uint32_t pollers) {
   unsigned l = lane_id();
-  uint32_t ns = 32;
+  uint32_t ns = 32, empty = 0;
   for (uint32_t iter = 0;; ++iter) {
     bool progress = false, lost = false;
     // device engine: serve one queue per iteration, one with work from a window of 32
-    // queues that rotates and differs between engines, so that every queue is visited
-    // often and commands do not wait behind long scans
+    // queues: its home queue first, which with every queue busy leaves few engines after
+    // the same commands, else one that rotates and differs between engines
     // (the doorbells and fetch counters of a window are two 128-byte lines read in one
     // round trip; they only select a queue, emu_serve checks them again.  Reading all
     // 128 queues in every pass of every engine kept those few lines so busy that the
@@ -1836,7 +1838,11 @@ static __device__ void service_loop(const Dev &d, uint32_t app_ctas, uint64_t de
       // without prefetch queues any window will do; with them every demand queue is
       // looked at before the first prefetch queue
       const uint32_t looks = d.Qp ? windows : 1u;
-      uint32_t w = windows == 1 ? 0u : (iter + sw) % windows;
+      // its home queue's window unless that was empty last time; every fourth look goes
+      // round all of them (more queues than engines)
+      const uint32_t home = sw % cnt;
+      const bool stray = (iter & 3) == 3;
+      uint32_t w = windows == 1 ? 0u : (stray ? (iter >> 2) + sw : (home >> 5) + empty) % windows;
       uint32_t qsel = ~0u, f = 0, db = 0;
       for (uint32_t k = 0; k < looks && qsel == ~0u; ++k) {
         const uint32_t off = w * 32 + l;
@@ -1848,13 +1854,16 @@ static __device__ void service_loop(const Dev &d, uint32_t app_ctas, uint64_t de
         unsigned m = __ballot_sync(kFull, (int32_t)(dbv - fv) > 0);
         if (m) {
           const uint32_t turn = ((sw * 31 + iter) * 0x9E3779B1u) >> 27;  // engines start at different queues
-          const int at = (__ffs(__funnelshift_r(m, m, turn)) - 1 + turn) & 31;
+          int at = (__ffs(__funnelshift_r(m, m, turn)) - 1 + turn) & 31;
+          if (!stray && w == home >> 5 && (m >> (home & 31)) & 1u) at = home & 31;
           qsel = base + w * 32 + at;
           f = __shfl_sync(kFull, fv, at);
           db = __shfl_sync(kFull, dbv, at);
         }
         if (++w == windows) w = 0;
       }
+      if (qsel == ~0u) ++empty;
+      else empty = 0;
       if (qsel != ~0u) {
         uint32_t r = emu_serve(d, qsel, f, db, block_dev);
         if (r == kEmuDevFull) block_dev = d.ndev > 1 ? qsel % d.ndev : 0u;
@@ -2015,9 +2024,24 @@ constexpr int engine_shared() {
   return SharedPerWarp<App>::value * EngineShape<App>::warps;
 }
 
+// An application with nothing to do says so with
+//   __device__ bool idle(const Dev &d) const;
+// (the same answer in every thread of the launch): its engine ends at once.
+template <class App, class = void>
+struct HasIdle {
+  static constexpr bool value = false;
+};
+template <class App>
+struct HasIdle<App, decltype((void)&App::idle)> {
+  static constexpr bool value = true;
+};
+
 template <class App>
 __global__ void __launch_bounds__(EngineShape<App>::threads, 1)
     engine_kernel(const __grid_constant__ Dev d, const __grid_constant__ App app) {
+  if constexpr (HasIdle<App>::value) {
+    if (app.idle(d)) return;
+  }
   constexpr uint32_t kCtaWarps = EngineShape<App>::warps;
   const Roles r = engine_roles(gridDim.x, kCtaWarps);
   // service CTAs are evenly spread over the grid
