@@ -371,7 +371,7 @@ struct PipeApp {
 
 // ============================================================================ BFS
 // Level-synchronous top-down BFS (Sec. 4.5 BFS over CSR, through the cache).
-// Level L: app warps claim chunks of 128 consecutive vertex ids; a lane owns one
+// Level L: app warps claim chunks of 32 to 128 consecutive vertex ids; a lane owns one
 // vertex and takes part when level[v] == L.  Its offsets[v], offsets[v+1] (int64) and
 // its neighbour list (int32) are read through the cache; every neighbour u with
 // level[u] == -1 gets level L+1 by compare-and-swap.  Vertices are visited in id order,
@@ -427,6 +427,11 @@ struct BfsAppT {
   HubEntry *hubq;
   uint32_t hub_cap;
   uint32_t *vis;  // visited bitmap: bit u set once level[u] is set (read through L1, may lag)
+  // vertices a warp claims at a time: kChunk, less when the graph has fewer than two such
+  // chunks for every warp (a chunk's units follow one another: 2^14 vertices on 256
+  // warps take 447 us with 128, 302 with 32; 2^20 vertices on 1,920 warps 2.79 ms with
+  // 128, 3.23 with 32, whose units wait for each other's pages)
+  uint32_t csize;
   const uint8_t *h_off = nullptr, *h_col = nullptr;  // kDirect: the CSR arrays in HBM
 
   static constexpr uint32_t kChunk = 128;
@@ -652,7 +657,7 @@ struct BfsAppT {
   // request (sparse levels): in dense ones the pages would outnumber what the cache
   // holds for the running warps.
   __device__ bool prefetch_chunk(const Dev &d, const AppCtx &a, uint32_t c0, uint32_t fbits, Pin &pc) const {
-    constexpr uint32_t U = kChunk / 32;
+    const uint32_t U = csize / 32;
     unsigned l = lane_id();
     // the lane's page to request (at most one over the chunk's units; two or more
     // anywhere in the warp: the chunk is not sparse, pages are requested when needed)
@@ -780,7 +785,7 @@ struct BfsAppT {
 
   __device__ void run(const Dev &d, const AppCtx &a) const {
     unsigned l = lane_id();
-    uint32_t nchunks = (n + kChunk - 1) / kChunk;
+    uint32_t nchunks = (n + csize - 1) / csize;
     unsigned long long scanned = 0;
     for (int32_t L = 0;; ++L) {
       if (a.warp == 0 && l == 0) {
@@ -804,20 +809,21 @@ struct BfsAppT {
         // the chunk's level words, all in flight together: bit k of fbits says whether
         // the lane's vertex of unit k is in the frontier (a word equal to L was written
         // at the level before and does not change during this one)
-        constexpr uint32_t U = kChunk / 32;
-        uint32_t lv[U];
+        constexpr uint32_t kUnits = kChunk / 32;
+        const uint32_t U = csize / 32, c0 = c * csize;
+        uint32_t lv[kUnits];
 #pragma unroll
-        for (uint32_t k = 0; k < U; ++k) {
-          uint32_t v = c * kChunk + 32 * k + l;
-          lv[k] = v < n ? ld_rlx32((const uint32_t *)&level[v]) : 0xFFFFFFFFu;
+        for (uint32_t k = 0; k < kUnits; ++k) {
+          uint32_t v = c0 + 32 * k + l;
+          lv[k] = k < U && v < n ? ld_rlx32((const uint32_t *)&level[v]) : 0xFFFFFFFFu;
         }
         uint32_t fbits = 0;
 #pragma unroll
-        for (uint32_t k = 0; k < U; ++k) fbits |= (lv[k] == (uint32_t)L ? 1u : 0u) << k;
+        for (uint32_t k = 0; k < kUnits; ++k) fbits |= (lv[k] == (uint32_t)L ? 1u : 0u) << k;
         if (!__any_sync(kFull, fbits)) continue;
-        if (!kDirect && mode == AGILE_ASYNC) ok = prefetch_chunk(d, a, c * kChunk, fbits, pc);
+        if (!kDirect && mode == AGILE_ASYNC) ok = prefetch_chunk(d, a, c0, fbits, pc);
         for (uint32_t k = 0; k < U && ok; ++k)
-          ok = chunk(d, a, c * kChunk + 32 * k, (fbits >> k) & 1u, L, found, scanned, pc);
+          ok = chunk(d, a, c0 + 32 * k, (fbits >> k) & 1u, L, found, scanned, pc);
         if (!ok) break;
       }
       // this warp queues no more slices of level L
@@ -849,15 +855,16 @@ using BfsApp = BfsAppT<false>;
 // ============================================================================ SpMV
 // y = A x over a CSR matrix on the store (Sec. 4.5 runs SpMV over the CSR graphs of its
 // BFS): int64 offsets, int32 columns and FP32 values are read through the cache; x and
-// y are device arrays of the caller.  Warps take chunks of kChunk consecutive rows, in
-// units of 32 rows (a lane owns a row); a unit's entries are flattened over the warp,
-// 32 a step, the column and the value of an entry each read through the cache.  The
-// offsets, column and value arrays each keep one pinned page; before a warp waits for a
-// page it lets the other two go, so it never waits while holding a pin.  A row's
-// products are added in increasing entry order: within a step by a chain over the
-// lanes (lane t adds its product to lane t-1's running sum), across steps through the
-// owner lane's running sum, so a row of fewer than kHub entries equals the sequential
-// definition bit for bit.  A row of at least kHub entries is queued as slices of
+// y are device arrays of the caller.  Warps take units of 32 consecutive rows (a lane
+// owns a row).  A unit's entries are multiplied in blocks of kSlice: flattened over the warp,
+// 128 a step, the columns, values and x of a step in flight together, the products into
+// shared memory; then every lane adds its own row's products of the block in entry order.
+// (Adding with a chain over the lanes took 31 dependent shuffles for 32 entries, and
+// a step of 32 entries three round trips: 4.5 ms for 31 M entries through a cache of an
+// eighth, 3.4 so.)  The offsets, column and value arrays each keep one pinned page; before a
+// warp waits for a page it lets the other two go, so it never waits while holding a pin.
+// A row of fewer than kHub entries so equals the sequential definition bit for bit.  A row of
+// at least kHub entries is queued as slices of
 // kSlice entries (the BFS slice queue), which any warp may take: the warp computes the
 // slice's products (into shared memory, all of its pages in flight together), then
 // takes the running sum the row's previous slice published (a slice waits for it
@@ -888,7 +895,9 @@ struct SpmvAppT {
   uint32_t hub_cap;
   const uint8_t *h_off = nullptr, *h_col = nullptr, *h_val = nullptr;  // kDirect: the CSR in HBM
 
-  static constexpr uint32_t kChunk = 128;
+  // rows a warp claims at a time: with 128 (four units) the claimed rows' pages were more
+  // than an eighth of the arrays and were evicted between units (101 k reads against 92 k)
+  static constexpr uint32_t kChunk = 32;
   static constexpr uint32_t kHub = 1024;
   static constexpr uint32_t kSlice = 1024;  // = the products buffer of a warp
   static constexpr int kSharedPerWarp = kSlice * 4;
@@ -971,34 +980,45 @@ struct SpmvAppT {
     }
   }
 
-  // product of the entry at `pos` (lanes with act): vals[pos] * x[cols[pos]], rounded
-  __device__ bool product(const Dev &d, const AppCtx &a, bool act, uint64_t pos, float &prod, Pin &po, Pin &pcol,
-                          Pin &pval) const {
-    const bool w[1] = {act};
-    const uint64_t b[1] = {pos * 4};
-    int32_t col[1] = {0};
-    float val[1] = {0.f};
-    if (!gather<int32_t, 1>(d, a, col_page0, w, b, col, pcol, pval, po)) return false;
-    if (!gather<float, 1>(d, a, val_page0, w, b, val, pval, pcol, po)) return false;
-    prod = 0.f;
-    if (act) {
-      float xv = 0.f;
-      if ((uint32_t)col[0] < n_x) xv = __ldg(&x[col[0]]);
-      else set_error(d, AGILE_EINVAL);
-      prod = __fmul_rn(val[0], xv);
+  // Products vals[pos] * x[cols[pos]], each rounded, of the N entries pos of the lanes (act).
+  template <int N>
+  __device__ bool products(const Dev &d, const AppCtx &a, const bool (&act)[N], const uint64_t (&pos)[N],
+                           float (&prod)[N], Pin &po, Pin &pcol, Pin &pval) const {
+    uint64_t b[N];
+    int32_t col[N];
+    float val[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      b[i] = pos[i] * 4;
+      col[i] = 0;
+      val[i] = 0.f;
     }
+    if (!gather<int32_t, N>(d, a, col_page0, act, b, col, pcol, pval, po)) return false;
+    if (!gather<float, N>(d, a, val_page0, act, b, val, pval, pcol, po)) return false;
+    float xv[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      xv[i] = 0.f;
+      if (act[i]) {
+        if ((uint32_t)col[i] < n_x) xv[i] = __ldg(&x[col[i]]);
+        else set_error(d, AGILE_EINVAL);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) prod[i] = __fmul_rn(val[i], xv[i]);
     return true;
   }
 
-  // In-order running sums over one step: unless it starts a row segment (its `run`
-  // already set by the caller), lane t adds its product to lane t-1's running sum.
-  __device__ __forceinline__ float chain(float run, float prod, bool cont) const {
-    unsigned l = lane_id();
+  // run + buf[i0] + ... + buf[i1 - 1], added in that order
+  __device__ __forceinline__ static float add_in_order(float run, const float *buf, uint32_t i0, uint32_t i1) {
+    for (; i0 + 8 <= i1; i0 += 8) {
+      float v[8];
 #pragma unroll
-    for (int t = 1; t < 32; ++t) {
-      float prev = __shfl_sync(kFull, run, t - 1);
-      if ((int)l == t && cont) run = __fadd_rn(prev, prod);
+      for (int k = 0; k < 8; ++k) v[k] = buf[i0 + k];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) run = __fadd_rn(run, v[k]);
     }
+    for (; i0 < i1; ++i0) run = __fadd_rn(run, buf[i0]);
     return run;
   }
 
@@ -1059,10 +1079,12 @@ struct SpmvAppT {
   }
 
   // The rows [v0, v0 + 32): lane l's row starts at entry s and has `dg` entries summed
-  // here (0 for a queued row): flattened over the warp, summed in order; y written for
-  // the lanes with `keep`.
+  // here (0 for a queued row, `holes`: there is one): y written for the lanes with `keep`.
   __device__ bool compute_unit(const Dev &d, const AppCtx &a, uint32_t v0, int64_t s, uint32_t dg, bool keep,
-                               Pin &po, Pin &pcol, Pin &pval) const {
+                               bool holes, Pin &po, Pin &pcol, Pin &pval) const {
+    extern __shared__ float prod_buf[];
+    float *buf = prod_buf + (threadIdx.x >> 5) * kSlice;
+    constexpr int N = 4;
     unsigned l = lane_id();
     uint32_t incl = dg;
 #pragma unroll
@@ -1072,32 +1094,44 @@ struct SpmvAppT {
     }
     uint32_t excl = incl - dg;
     uint32_t total = __shfl_sync(kFull, incl, 31);
+    // without holes entry k of the unit is entry first + k of the matrix
+    const int64_t first = __shfl_sync(kFull, s, 0);
     float acc = 0.0f;  // this lane's row: running sum
-    for (uint32_t k0 = 0; k0 < total; k0 += 32) {
-      uint32_t k = k0 + l;
-      bool act = k < total;
-      // owner lane j: the last lane whose exclusive prefix is <= k
-      uint32_t j = 0;
+    for (uint32_t b0 = 0; b0 < total; b0 += kSlice) {
+      const uint32_t m = min(kSlice, total - b0);
+      for (uint32_t k0 = 0; k0 < m; k0 += 32 * N) {
+        bool act[N];
+        uint64_t pos[N];
+        float prod[N];
 #pragma unroll
-      for (int step = 16; step >= 1; step >>= 1) {
-        uint32_t cand = j + step;
-        uint32_t ex = __shfl_sync(kFull, excl, cand & 31);
-        if (cand < 32 && ex <= k) j = cand;
+        for (int h = 0; h < N; ++h) {
+          const uint32_t kb = k0 + 32 * h + l, k = b0 + kb;
+          act[h] = kb < m;
+          if (!holes) {
+            pos[h] = act[h] ? (uint64_t)first + k : 0;
+            continue;
+          }
+          // owner lane j: the last lane whose exclusive prefix is <= k
+          uint32_t j = 0;
+#pragma unroll
+          for (int step = 16; step >= 1; step >>= 1) {
+            uint32_t cand = j + step;
+            uint32_t ex = __shfl_sync(kFull, excl, cand & 31);
+            if (cand < 32 && ex <= k) j = cand;
+          }
+          int64_t sj = __shfl_sync(kFull, s, j);
+          uint32_t exj = __shfl_sync(kFull, excl, j);
+          pos[h] = act[h] ? (uint64_t)sj + (k - exj) : 0;
+        }
+        if (!products<N>(d, a, act, pos, prod, po, pcol, pval)) return false;
+#pragma unroll
+        for (int h = 0; h < N; ++h)
+          if (act[h]) buf[k0 + 32 * h + l] = prod[h];
       }
-      int64_t sj = __shfl_sync(kFull, s, j);
-      uint32_t exj = __shfl_sync(kFull, excl, j);
-      float prod = 0.f;
-      if (!product(d, a, act, act ? (uint64_t)sj + (k - exj) : 0, prod, po, pcol, pval)) return false;
-      float carry = __shfl_sync(kFull, acc, j);
-      bool first = act && (k == exj || l == 0);  // the row's first entry in this step
-      float run = first ? __fadd_rn(k == exj ? 0.0f : carry, prod) : prod;
-      run = chain(run, prod, act && !first);
-      // the owner takes its row's running sum from the row's last lane in this step
-      uint32_t endk = excl + dg;
-      bool mine = dg > 0 && excl < k0 + 32 && endk > k0;
-      uint32_t last = mine ? min(endk, k0 + 32) - 1 - k0 : 0;
-      float got = __shfl_sync(kFull, run, last);
-      if (mine) acc = got;
+      __syncwarp();
+      const uint32_t i0 = max(excl, b0), i1 = min(excl + dg, b0 + m);
+      if (i0 < i1) acc = add_in_order(acc, buf, i0 - b0, i1 - b0);
+      __syncwarp();
     }
     if (keep) y[v0 + l] = acc;
     return true;
@@ -1118,7 +1152,7 @@ struct SpmvAppT {
 
   // ASYNC: read the unit's offsets, queue its long rows, request its column and value pages
   __device__ bool issue_unit(const Dev &d, const AppCtx &a, uint32_t v0, int64_t &s, uint32_t &dg, bool &keep,
-                             unsigned long long &entries, Pin &po, Pin &pcol, Pin &pval) const {
+                             bool &holes, unsigned long long &entries, Pin &po, Pin &pcol, Pin &pval) const {
     uint32_t v = v0 + lane_id();
     bool f = v < n;
     int64_t e = 0;
@@ -1129,8 +1163,22 @@ struct SpmvAppT {
     bool hub = push_hub(d, v, deg, s, e);
     dg = hub ? 0 : deg;
     keep = f && !hub;
-    // the entries summed here lie in one span (queued rows are holes in it): request
-    // the span's pages of both arrays, at most 32 of each
+    holes = __any_sync(kFull, hub);
+    if (!kDirect && holes) {
+      // the pages of the lanes' own rows (at most two each), not those of the queued rows
+      // between them, which are read with their slices
+      const uint64_t p0 = ((uint64_t)s * 4) / kPage, p1 = dg ? ((uint64_t)(s + dg - 1) * 4) / kPage : p0;
+      const uint64_t arr[2] = {col_page0, val_page0};
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        if (!warp_request_call(d, dg != 0, arr[k] + p0, a.q0, false, a.deadline, true)) return false;
+        if (__any_sync(kFull, p1 != p0) &&
+            !warp_request_call(d, p1 != p0, arr[k] + p1, a.q0, false, a.deadline, true))
+          return false;
+      }
+      return true;
+    }
+    // the unit's entries lie in one span: request its pages of both arrays, at most 32 of each
     long long lo = dg ? s : LLONG_MAX, hi = dg ? s + dg : 0;
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) {
@@ -1146,7 +1194,7 @@ struct SpmvAppT {
 
   // take queued slices until every slice is taken (the BFS slice queue, one level)
   __device__ bool help_hubs(const Dev &d, const AppCtx &a, Pin &po, Pin &pcol, Pin &pval) const {
-    extern __shared__ float prod_buf[];  // products of the slice a warp holds
+    extern __shared__ float prod_buf[];  // products of the slice a warp holds (kSlice a warp)
     float *buf = prod_buf + (threadIdx.x >> 5) * kSlice;
     unsigned l = lane_id();
     const uint64_t ep = launch_epoch(d);
@@ -1200,29 +1248,22 @@ struct SpmvAppT {
         if (!warp_request_call(d, want, col_page0 + c0 + l, a.q0, false, a.deadline)) return false;
         if (!warp_request_call(d, want, val_page0 + c0 + l, a.q0, false, a.deadline)) return false;
       }
-      // products of the slice, two entries a lane at a time, into the warp's buffer
-      for (int64_t b0 = p0; b0 < p1; b0 += 64) {
-        bool on[2];
-        uint64_t byte[2];
-        int32_t col[2] = {0, 0};
-        float val[2] = {0.f, 0.f};
+      // products of the slice, four entries a lane at a time, into the warp's buffer
+      constexpr int N = 4;
+      for (int64_t b0 = p0; b0 < p1; b0 += 32 * N) {
+        bool on[N];
+        uint64_t pos[N];
+        float prod[N];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          int64_t pos = b0 + 32 * h + l;
-          on[h] = pos < p1;
-          byte[h] = (uint64_t)(on[h] ? pos : p0) * 4;
+        for (int h = 0; h < N; ++h) {
+          pos[h] = (uint64_t)(b0 + 32 * h + l);
+          on[h] = (int64_t)pos[h] < p1;
+          if (!on[h]) pos[h] = (uint64_t)p0;
         }
-        if (!gather<int32_t, 2>(d, a, col_page0, on, byte, col, pcol, pval, po)) return false;
-        if (!gather<float, 2>(d, a, val_page0, on, byte, val, pval, pcol, po)) return false;
+        if (!products<N>(d, a, on, pos, prod, po, pcol, pval)) return false;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (on[h]) {
-            float xv = 0.f;
-            if ((uint32_t)col[h] < n_x) xv = __ldg(&x[col[h]]);
-            else set_error(d, AGILE_EINVAL);
-            buf[b0 - p0 + 32 * h + l] = __fmul_rn(val[h], xv);
-          }
-        }
+        for (int h = 0; h < N; ++h)
+          if (on[h]) buf[pos[h] - (uint64_t)p0] = prod[h];
       }
       // the running sum of the row so far: +0 before its first entry, else what the
       // previous slice (the record before this one) published; waited for holding no pin
@@ -1247,8 +1288,7 @@ struct SpmvAppT {
       }
       __syncwarp();
       if (l == 0) {
-        const uint32_t cnt = (uint32_t)(p1 - p0);
-        for (uint32_t i = 0; i < cnt; ++i) run = __fadd_rn(run, buf[i]);
+        run = add_in_order(run, buf, 0, (uint32_t)(p1 - p0));
         if (last) y[row] = run;
         else st_rel64(&r->carry, (ep << 32) | __float_as_uint(run));
       }
@@ -1268,9 +1308,9 @@ struct SpmvAppT {
       while (ok && next_unit(d, nchunks, chunk, sub, v0)) {
         int64_t s = 0;
         uint32_t dg = 0;
-        bool k = false;
-        ok = issue_unit(d, a, v0, s, dg, k, entries, po, pcol, pval);
-        if (ok) ok = compute_unit(d, a, v0, s, dg, k, po, pcol, pval);
+        bool k = false, holes = false;
+        ok = issue_unit(d, a, v0, s, dg, k, holes, entries, po, pcol, pval);
+        if (ok) ok = compute_unit(d, a, v0, s, dg, k, holes, po, pcol, pval);
       }
     } else {
       uint32_t v0 = 0;
@@ -1283,7 +1323,7 @@ struct SpmvAppT {
         uint32_t deg = f ? (uint32_t)(e - s) : 0;
         entries += __reduce_add_sync(kFull, deg);
         bool hub = push_hub(d, v, deg, s, e);
-        ok = compute_unit(d, a, v0, s, hub ? 0 : deg, f && !hub, po, pcol, pval);
+        ok = compute_unit(d, a, v0, s, hub ? 0 : deg, f && !hub, __any_sync(kFull, hub), po, pcol, pval);
       }
     }
     // this warp queues no more slices
@@ -1550,18 +1590,22 @@ int bfs_launch(agile_ctx *c, uint64_t offsets_byte0, uint64_t cols_byte0, uint32
   bfs_init_kernel<<<(n_vertices + 255) / 256, 256, 0, s>>>(d_level, vis, n_vertices, src);
   AGILE_CUDA_TRY(cudaGetLastError());
   if (d_edges_scanned) AGILE_CUDA_TRY(cudaMemsetAsync(d_edges_scanned, 0, 8, s));
+  // about two lines per warp (one pinned, one being filled; a slice's requested pages are
+  // scanned right away)
+  const uint32_t warps = warps_for_cache(c, 2, 32);
+  const uint32_t run = running_app_warps<BfsApp>(c, warps);
+  uint32_t csize = BfsApp::kChunk;
+  while (csize > 32 && n_vertices / csize < 2 * run) csize /= 2;
   if (h_off) {
     // the CSR in HBM: offsets and columns are told apart by their (distinct) page
     // numbers 0 and 1 only
     BfsAppT<true> app{0, 1, n_vertices, d_level, (unsigned long long *)d_edges_scanned, AGILE_SYNC, hubq,
-                      hub_cap, vis, (const uint8_t *)h_off, (const uint8_t *)h_col};
-    return launch_engine(c, app, stream, warps_for_cache(c, 2, 32));
+                      hub_cap, vis, csize, (const uint8_t *)h_off, (const uint8_t *)h_col};
+    return launch_engine(c, app, stream, warps);
   }
   BfsApp app{offsets_byte0 / kPage, cols_byte0 / kPage, n_vertices, d_level,
-             (unsigned long long *)d_edges_scanned, mode, hubq, hub_cap, vis};
-  // about two lines per warp (one pinned, one being filled; a slice's requested pages are
-  // scanned right away)
-  return launch_engine(c, app, stream, warps_for_cache(c, 2, 32));
+             (unsigned long long *)d_edges_scanned, mode, hubq, hub_cap, vis, csize};
+  return launch_engine(c, app, stream, warps);
 }
 
 // ---------------------------------------------------------------- BFS without allocation
@@ -1875,8 +1919,8 @@ int agile_spmv(agile_ctx *c, uint64_t offsets_byte0, uint64_t cols_byte0, uint64
   if (d_entries) AGILE_CUDA_TRY(cudaMemsetAsync(d_entries, 0, 8, as_stream(stream)));
   SpmvApp app{offsets_byte0 / kPage, cols_byte0 / kPage, vals_byte0 / kPage, n_rows, d_x, n_cols, d_y,
               (unsigned long long *)d_entries, mode, (HubEntry *)c->bfs_hubq, c->bfs_hub_cap};
-  // each warp pins one page of each of three arrays and requests up to two units ahead
-  return launch_engine(c, app, stream, warps_for_cache(c, mode == AGILE_ASYNC ? 6 : 3, 32));
+  // each warp pins one page of each of three arrays and requests a unit's (two of each)
+  return launch_engine(c, app, stream, warps_for_cache(c, mode == AGILE_ASYNC ? 4 : 3, 32));
 }
 
 }  // extern "C"

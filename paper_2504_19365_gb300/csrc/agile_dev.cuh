@@ -855,8 +855,11 @@ static __device__ __forceinline__ int cache_claim(const Dev &d, uint64_t page, u
     c.w0 = sq_first_word(d, q0, dev_of_page(d, page), pf);
     c.sh = sh_insert(d, page, SH_FILL);
     if (c.sh < 0) {
+      // another thread is at the page (a request made without waiting is done with it) or
+      // the bucket is full
       atomicAdd(stat_ptr(d, S_SHARE_RETRIES), 1ull);
-      return M_RETRY;
+      c.line = 0;
+      return c.sh == -1 ? M_BUSY : M_RETRY;
     }
   }
   const uint32_t set = set_of(page, d.sets);
