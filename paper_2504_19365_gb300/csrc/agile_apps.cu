@@ -192,8 +192,16 @@ struct EmbApp {
     constexpr int RB = MF4 >= 8 ? 1 : 8 / MF4;  // rows of an all-resident bag loaded before the next probe
     Prep cur;
     prep(d, a.warp, cur);
-    for (uint32_t b = a.warp; b < n_bags; b += a.n_warps) {
-      uint32_t nb = b + a.n_warps;
+    // the lookahead walks the warp's own bags, so they are fixed; without one a warp takes
+    // the next bag that is left (bags differ in rows and in how many of them miss)
+    auto after = [&](uint32_t b) -> uint32_t {
+      if (async) return b + a.n_warps;
+      uint32_t k = 0;
+      if (l == 0) k = atomicAdd(&d.run->work[0], 1u);
+      return a.n_warps + __shfl_sync(kFull, k, 0);
+    };
+    for (uint32_t b = a.warp, nb; b < n_bags; b = nb) {
+      nb = after(b);
       if (!(cur.fast && cur.ok)) {
         // nothing pinned: the general path may wait
         if (async && cur.fast && !issue_rows(d, a, pf, cur.cnt, bo)) return;

@@ -481,10 +481,13 @@ static __device__ __forceinline__ void sq_ring(const Dev &d, uint32_t q, uint32_
     for (uint32_t k = 0; k < n; ++k)
       st_rlx64(&st[(ticket + k) & d.dmask], ((uint64_t)(ticket + k) << 2) | SQE_UPDATED);
     fence_sc();
-    uint32_t old = atomicCAS(db, ticket, ticket + n);
-    // the issuer before us may have seen the first mark and not yet the second
-    if (n == 2 && old == ticket + 1 && atomicCAS(db, ticket + 1, ticket + 2) == ticket + 1) old = ticket;
-    if (old != ticket) return;
+    uint32_t from = ticket, old = atomicCAS(db, from, ticket + n);
+    // the issuer before us may have seen the first marks and not yet the others
+    while (old != from && old - ticket < n) {
+      from = old;
+      old = atomicCAS(db, from, ticket + n);
+    }
+    if (old != from) return;
   }
   for (uint32_t t = ticket + n;;) {
     ++rung;
@@ -497,6 +500,37 @@ static __device__ __forceinline__ void sq_ring(const Dev &d, uint32_t q, uint32_
     t += m;
   }
   atomicAdd(stat_ptr(d, S_DOORBELLS), (unsigned long long)rung);
+}
+
+// Warp-collective reservation for lanes that need one slot each: the lanes with `want` of
+// an aligned group of four share one compare-and-swap on their first lane's queue and
+// take consecutive slots, and that lane rings for them all (`n` commands from `first` on;
+// n = 0 in the others).  Four, not the whole warp: engines take the commands of one queue
+// two at a time, a round trip each.  For bursts, where the threads' compare-and-swaps on a
+// queue's two words bound its issue (a flush of 8 k lines, 64 a queue: the last command was
+// written 192 us after the first, 96 with groups; the few misses of a lookup or a scan are
+// slower with it, 3 %).  For one device only (consecutive slots of a queue).
+// False for a lane of a group that found no room.
+static __device__ __forceinline__ bool sq_reserve_group(const Dev &d, bool want, uint32_t q0, uint32_t &q,
+                                                        uint32_t &slot, uint32_t &ticket, uint32_t &first, uint32_t &n,
+                                                        bool pf = false, uint64_t w0 = kNoWord) {
+  const unsigned l = lane_id(), base = l & ~3u;
+  const uint32_t mine = (__ballot_sync(kFull, want) >> base) & 15u;
+  const int lead = (int)base + (mine ? __ffs(mine) - 1 : 0);
+  bool ok = false;
+  n = 0;
+  if (want && lead == (int)l) {
+    n = __popc(mine);
+    ok = sq_reserve_dev(d, q0, 0, n, q, slot, ticket, pf, w0);
+  }
+  __syncwarp();
+  ok = __shfl_sync(kFull, ok, lead);
+  q = __shfl_sync(kFull, q, lead);
+  first = __shfl_sync(kFull, ticket, lead);
+  ticket = first + __popc(mine & ((1u << (l & 3)) - 1));
+  slot = ticket & d.dmask;
+  if (!ok) n = 0;
+  return ok && want;
 }
 
 // ================================================================ in-flight share table
@@ -1043,39 +1077,41 @@ static __device__ __noinline__ Requested warp_request_body(bool want, uint64_t p
         dropped = true;
       }
     }
-    if (missed) {
-      m = cache_claim(d, page, q0, c, true, -1, pf);
-      if (m != M_RETRY) line = c.line;
-    }
-    __syncwarp();
-    if (m == M_ISSUED) m = cache_reserve(d, page, q0, c, pf);
-    // MODIFIED victims are copied to their staging pages by the whole warp
-    for (unsigned wb = __ballot_sync(kFull, m == M_ISSUED && c.wb); wb; wb &= wb - 1) {
-      const int j = __ffs(wb) - 1;
-      const uint64_t src = __shfl_sync(kFull, (uint64_t)line_ptr(d, c.line), j);
-      const uint64_t dst = __shfl_sync(kFull, (uint64_t)claim_staging(d, c), j);
-      warp_copy_page((void *)dst, (const void *)src);
-    }
-    __syncwarp();
-    if (missed) {
-      if (m == M_ISSUED) {
-        Issued is;
-        cache_issue(d, page, c, is);
-        sent = true;
-        tok = ((uint64_t)is.q << 48) | ((uint64_t)is.slot << 32) | is.ticket;
-        code = is.code;
-        if (!wait) need = false;
-      } else if (m == M_HIT) {
-        need = false;
-      } else if (m == M_BUSY) {
-        if (!wait) need = false;
-      } else if (!wait && (hint || ++retries >= 4)) {
-        need = false;  // a prefetch is a hint: give up when nothing can be evicted now
-        if (hint) dropped = true;
+    if (__any_sync(kFull, missed)) {
+      if (missed) {
+        m = cache_claim(d, page, q0, c, true, -1, pf);
+        if (m != M_RETRY) line = c.line;
       }
+      __syncwarp();
+      if (m == M_ISSUED) m = cache_reserve(d, page, q0, c, pf);
+      // MODIFIED victims are copied to their staging pages by the whole warp
+      for (unsigned wb = __ballot_sync(kFull, m == M_ISSUED && c.wb); wb; wb &= wb - 1) {
+        const int j = __ffs(wb) - 1;
+        const uint64_t src = __shfl_sync(kFull, (uint64_t)line_ptr(d, c.line), j);
+        const uint64_t dst = __shfl_sync(kFull, (uint64_t)claim_staging(d, c), j);
+        warp_copy_page((void *)dst, (const void *)src);
+      }
+      __syncwarp();
+      if (missed) {
+        if (m == M_ISSUED) {
+          Issued is;
+          cache_issue(d, page, c, is);
+          sent = true;
+          tok = ((uint64_t)is.q << 48) | ((uint64_t)is.slot << 32) | is.ticket;
+          code = is.code;
+          if (!wait) need = false;
+        } else if (m == M_HIT) {
+          need = false;
+        } else if (m == M_BUSY) {
+          if (!wait) need = false;
+        } else if (!wait && (hint || ++retries >= 4)) {
+          need = false;  // a prefetch is a hint: give up when nothing can be evicted now
+          if (hint) dropped = true;
+        }
+      }
+      __syncwarp();
     }
     first = false;
-    __syncwarp();
     if (__any_sync(kFull, need)) {
       if (need) {
         if (gtimer() > deadline || aborted(d)) {

@@ -42,7 +42,7 @@ __global__ void bag_of_kernel(const int64_t *off, uint32_t n_bags, int32_t *bag_
 // __match_any_sync, so equal digits keep their order: no key needs its position to be
 // told apart, and the low word carries the bag instead.  Bound by launch latency at a
 // training batch's size (three passes of ~2 us a launch): 81,920 positions of 2^18 rows
-// take 18 us of kernels; the bitonic network it replaces took 153 launches, 263 us.
+// take 25 us of kernels; the bitonic network it replaces took 153 launches, 263 us.
 constexpr int kSortThreads = 256, kSortWarps = kSortThreads / 32;
 
 struct SortIn {  // where a pass reads its keys: the caller's indices (first pass) or the last pass's output
@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(SortIn in, u
 // can hide is the loads: the warp stages its 128-byte pieces of 32 gradient rows at a time
 // in shared memory with cp.async, three stages ahead of the adds (the keys one more), and
 // a wide row is shared by dim / 32 warps.  The 10 k positions of the hottest row (2^18
-// rows, Zipf 1.1, batch 4096 x 20) were 4.1 ms of serial load latency in one engine warp;
-// the bound that is left is the chain (4 cycles an add, 20 us).
+// rows, Zipf 1.1, batch 4096 x 20) were 4.1 ms of serial load latency in one engine warp and
+// take 119 us here; the bound that is left is the chain (4 cycles an add, 20 us).
 constexpr uint32_t kLong = 64;
 constexpr int kStages = 4, kLongWarps = 2;
 
@@ -210,15 +210,29 @@ __global__ void __launch_bounds__(32 * kLongWarps) long_rows_kernel(const uint64
   if (j0 == ~0ull) return;
   const uint32_t r = (uint32_t)(keys[j0] >> 32);
   const uint32_t per = 32 / nc;  // rows one warp-wide copy brings
-  // positions of batch b that belong to the row (a prefix: the keys are sorted), their bags
-  auto fetch = [&](uint64_t b, uint32_t &bag) -> uint32_t {
+  // a batch is 32 positions; those of the row are a prefix of it (the keys are sorted).
+  // Its keys are loaded one batch before they are looked at, so that no load is waited for
+  // in the loop.
+  auto keys_of = [&](uint64_t b) -> uint64_t {
     uint64_t j = j0 + 32 * b + l;
-    uint64_t key = j < n ? keys[j] : ~0ull;
-    bag = (uint32_t)key;
-    return __popc(__ballot_sync(kFull, j < n && (uint32_t)(key >> 32) == r));
+    return j < n ? keys[j] : ~((uint64_t)r << 32);  // past the end: another row
   };
+  auto count = [&](uint64_t key) -> uint32_t { return __popc(__ballot_sync(kFull, (uint32_t)(key >> 32) == r)); };
   auto copy = [&](uint64_t b, uint32_t bag, uint32_t c) {
     float *s = stage[w][b % kStages];
+    if (c == 32 && nc == 8) {  // a whole batch of 128-byte pieces: four rows a copy, no loop
+      const float *src = gout + col0 + 4 * (l & 7);
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s + (l >> 3) * 32 + 4 * (l & 7));
+      uint32_t bi[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) bi[t] = __shfl_sync(kFull, bag, 4 * t + (l >> 3));
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 512 * t), "l"(src + (uint64_t)bi[t] * dim)
+                     : "memory");
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      return;
+    }
     for (uint32_t i0 = 0; i0 < c; i0 += per) {
       uint32_t i = i0 + l / nc;
       uint32_t bi = __shfl_sync(kFull, bag, i & 31);
@@ -230,13 +244,16 @@ __global__ void __launch_bounds__(32 * kLongWarps) long_rows_kernel(const uint64
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  uint32_t cnt[kStages], bag_next, c_next = fetch(0, bag_next);
+  uint32_t cnt[kStages];
+  uint64_t key[kStages];
+#pragma unroll
+  for (int b = 0; b < kStages; ++b) key[b] = keys_of(b);
 #pragma unroll
   for (int b = 0; b < kStages - 1; ++b) {
-    cnt[b] = c_next;
-    copy(b, bag_next, c_next);
-    c_next = fetch(b + 1, bag_next);
+    cnt[b] = count(key[b]);
+    copy(b, (uint32_t)key[b], cnt[b]);
   }
+  uint64_t next = key[kStages - 1];
   float acc = 0.0f;
   for (uint64_t b0 = 0;; b0 += kStages) {
 #pragma unroll
@@ -244,15 +261,19 @@ __global__ void __launch_bounds__(32 * kLongWarps) long_rows_kernel(const uint64
       const uint64_t b = b0 + k;
       const int ahead = (k + kStages - 1) % kStages;
       // the stage being refilled was summed one batch ago
-      cnt[ahead] = c_next;
-      copy(b + kStages - 1, bag_next, c_next);
-      c_next = fetch(b + kStages, bag_next);
+      const uint64_t now = next;
+      next = keys_of(b + kStages);
+      cnt[ahead] = count(now);
+      copy(b + kStages - 1, (uint32_t)now, cnt[ahead]);
       asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 1) : "memory");
       __syncwarp();
       const float *s = stage[w][k] + (l < wide ? l : 0);
-      if (cnt[k] == 32) {
+      if (cnt[k] == 32 && nc == 8) {
+        float v[32];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) acc = __fadd_rn(acc, s[i * wide]);
+        for (int i = 0; i < 32; ++i) v[i] = s[i * 32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) acc = __fadd_rn(acc, v[i]);
       } else {
         for (uint32_t i = 0; i < cnt[k]; ++i) acc = __fadd_rn(acc, s[i * wide]);
       }
