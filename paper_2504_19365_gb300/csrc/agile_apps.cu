@@ -440,6 +440,10 @@ struct BfsAppT {
   // warps take 447 us with 128, 302 with 32; 2^20 vertices on 1,920 warps 2.79 ms with
   // 128, 3.23 with 32, whose units wait for each other's pages)
   uint32_t csize;
+  // ... and at a level with few vertices (under 1 in 256), where a claim is mostly a look at
+  // the level words: as many as leave a claim for every warp (2^20 vertices: 512; a near-empty
+  // level took 22 us of claims)
+  uint32_t wide;
   const uint8_t *h_off = nullptr, *h_col = nullptr;  // kDirect: the CSR arrays in HBM
 
   static constexpr uint32_t kChunk = 128;
@@ -664,8 +668,7 @@ struct BfsAppT {
   // instead of following one another.  Only when each lane has at most one page to
   // request (sparse levels): in dense ones the pages would outnumber what the cache
   // holds for the running warps.
-  __device__ bool prefetch_chunk(const Dev &d, const AppCtx &a, uint32_t c0, uint32_t fbits, Pin &pc) const {
-    const uint32_t U = csize / 32;
+  __device__ bool prefetch_chunk(const Dev &d, const AppCtx &a, uint32_t c0, uint32_t U, uint32_t fbits, Pin &pc) const {
     unsigned l = lane_id();
     // the lane's page to request (at most one over the chunk's units; two or more
     // anywhere in the warp: the chunk is not sparse, pages are requested when needed)
@@ -727,9 +730,8 @@ struct BfsAppT {
   // Take queued slices of level L, one ticket (a record index) at a time, until every
   // slice is taken.  A ticket waits, holding no pin, for its record to be published;
   // it is past the last slice when every warp has finished its own vertices (no more
-  // reservations come) and the reserved count is at most the ticket.  Each warp so ends
-  // with one ticket past the last slice.  Waiting warps watch their own record and look
-  // at the shared counters only now and then.
+  // reservations come) and the reserved count is at most the ticket (slices_end).  Each warp
+  // so ends with one ticket past the last slice.
   __device__ bool help_hubs(const Dev &d, const AppCtx &a, int32_t L, uint32_t &found, Pin &pc) const {
     unsigned l = lane_id();
     const uint64_t want_tag = tag(d, L);
@@ -742,12 +744,11 @@ struct BfsAppT {
       HubEntry *r = &hubq[k];
       uint32_t ns = 64;
       int state = 0;  // 1: record published, 2: past the last slice
-      for (uint32_t spin = 0;; ++spin) {
+      for (;;) {
         if (l == 0) {
           if (ld_acq64(&r->ready) == want_tag) {
             state = 1;
-          } else if ((spin & 7) == 7 && ld_acq32(&d.run->units_done[par]) >= a.n_warps &&
-                     ld_acq32(&d.run->hub_count[par]) <= k) {
+          } else if (slices_end(d, par, (uint32_t)L, k)) {
             state = 2;
           }
         }
@@ -758,7 +759,7 @@ struct BfsAppT {
           if (l == 0) set_error(d, -110);
           return false;
         }
-        backoff(ns, 1024);
+        backoff(ns, 256);
       }
       if (state == 2) return true;
       int64_t p0 = 0, p1 = 0;
@@ -793,7 +794,7 @@ struct BfsAppT {
 
   __device__ void run(const Dev &d, const AppCtx &a) const {
     unsigned l = lane_id();
-    uint32_t nchunks = (n + csize - 1) / csize;
+    uint64_t frontier = 1;  // vertices of the level
     unsigned long long scanned = 0;
     for (int32_t L = 0;; ++L) {
       if (a.warp == 0 && l == 0) {
@@ -809,16 +810,23 @@ struct BfsAppT {
       uint32_t found = 0;
       Pin pc{0, 0, false};
       bool ok = true;
-      for (;;) {
-        uint32_t c = 0;
-        if (l == 0) c = atomicAdd(&d.run->work[L & 1], 1u);
-        c = __shfl_sync(kFull, c, 0);
-        if (c >= nchunks || aborted(d)) break;
+      const uint32_t span = frontier * 256 < n ? wide : csize, step = min(span, kChunk), U = step / 32;
+      const uint32_t nchunks = (uint32_t)(((uint64_t)n + span - 1) / span);
+      uint32_t c = 0, at = span;  // the claimed chunk and how far the warp is in it
+      for (; ok; at += step) {
+        if (at >= span) {
+          if (l == 0) c = atomicAdd(&d.run->work[L & 1], 1u);
+          c = __shfl_sync(kFull, c, 0);
+          if (c >= nchunks || aborted(d)) break;
+          at = 0;
+        }
+        const uint64_t v00 = (uint64_t)c * span + at;
+        if (v00 >= n) continue;
+        const uint32_t c0 = (uint32_t)v00;
         // the chunk's level words, all in flight together: bit k of fbits says whether
         // the lane's vertex of unit k is in the frontier (a word equal to L was written
         // at the level before and does not change during this one)
         constexpr uint32_t kUnits = kChunk / 32;
-        const uint32_t U = csize / 32, c0 = c * csize;
         uint32_t lv[kUnits];
 #pragma unroll
         for (uint32_t k = 0; k < kUnits; ++k) {
@@ -829,16 +837,14 @@ struct BfsAppT {
 #pragma unroll
         for (uint32_t k = 0; k < kUnits; ++k) fbits |= (lv[k] == (uint32_t)L ? 1u : 0u) << k;
         if (!__any_sync(kFull, fbits)) continue;
-        if (!kDirect && mode == AGILE_ASYNC) ok = prefetch_chunk(d, a, c0, fbits, pc);
+        if (!kDirect && mode == AGILE_ASYNC) ok = prefetch_chunk(d, a, c0, U, fbits, pc);
         for (uint32_t k = 0; k < U && ok; ++k)
           ok = chunk(d, a, c0 + 32 * k, (fbits >> k) & 1u, L, found, scanned, pc);
-        if (!ok) break;
       }
       // this warp queues no more slices of level L
       __syncwarp();
       if (l == 0) {
-        fence_ar();
-        atomicAdd(&d.run->units_done[L & 1], 1u);
+        own_work_done(d, L & 1);
         app_event(d, a.warp, kEvOwnDone, (uint32_t)L);
       }
       if (ok) help_hubs(d, a, L, found, pc);
@@ -851,6 +857,7 @@ struct BfsAppT {
       if (aborted(d)) return;
       uint64_t disc = ld_acq64(&d.run->acc[1 + L % 3]);
       if (disc == 0) break;
+      frontier = disc;
     }
     if (l == 0 && scanned) atomicAdd(&d.run->acc[0], scanned);
     if (!app_barrier(d, a.n_warps, a.deadline)) return;
@@ -1215,12 +1222,11 @@ struct SpmvAppT {
       HubEntry *r = &hubq[k];
       uint32_t ns = 64;
       int state = 0;  // 1: record published, 2: past the last slice
-      for (uint32_t spin = 0;; ++spin) {
+      for (;;) {
         if (l == 0) {
           if (ld_acq64(&r->ready) == want_tag) {
             state = 1;
-          } else if ((spin & 7) == 7 && ld_acq32(&d.run->units_done[0]) >= a.n_warps &&
-                     ld_acq32(&d.run->hub_count[0]) <= k) {
+          } else if (slices_end(d, 0, 0, k)) {
             state = 2;
           }
         }
@@ -1233,7 +1239,7 @@ struct SpmvAppT {
           if (l == 0) set_error(d, -110);
           return false;
         }
-        backoff(ns, 1024);
+        backoff(ns, 256);
       }
       if (state == 2) return true;
       int64_t p0 = 0, p1 = 0;
@@ -1336,10 +1342,7 @@ struct SpmvAppT {
     }
     // this warp queues no more slices
     __syncwarp();
-    if (l == 0) {
-      fence_ar();
-      atomicAdd(&d.run->units_done[0], 1u);
-    }
+    if (l == 0) own_work_done(d, 0);
     if (ok) help_hubs(d, a, po, pcol, pval);
     release(d, po);
     release(d, pcol);
@@ -1604,15 +1607,17 @@ int bfs_launch(agile_ctx *c, uint64_t offsets_byte0, uint64_t cols_byte0, uint32
   const uint32_t run = running_app_warps<BfsApp>(c, warps);
   uint32_t csize = BfsApp::kChunk;
   while (csize > 32 && n_vertices / csize < 2 * run) csize /= 2;
+  uint32_t wide = BfsApp::kChunk;
+  while (wide < 1024 && n_vertices / (2 * wide) >= run) wide *= 2;
   if (h_off) {
     // the CSR in HBM: offsets and columns are told apart by their (distinct) page
     // numbers 0 and 1 only
     BfsAppT<true> app{0, 1, n_vertices, d_level, (unsigned long long *)d_edges_scanned, AGILE_SYNC, hubq,
-                      hub_cap, vis, csize, (const uint8_t *)h_off, (const uint8_t *)h_col};
+                      hub_cap, vis, csize, wide, (const uint8_t *)h_off, (const uint8_t *)h_col};
     return launch_engine(c, app, stream, warps);
   }
   BfsApp app{offsets_byte0 / kPage, cols_byte0 / kPage, n_vertices, d_level,
-             (unsigned long long *)d_edges_scanned, mode, hubq, hub_cap, vis, csize};
+             (unsigned long long *)d_edges_scanned, mode, hubq, hub_cap, vis, csize, wide};
   return launch_engine(c, app, stream, warps);
 }
 

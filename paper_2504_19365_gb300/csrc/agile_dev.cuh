@@ -82,7 +82,7 @@ struct RunState {
   // BFS slice queue, per level parity, each on a line of its own (hot words)
   alignas(128) uint32_t hub_count[2];  // slices of long adjacency lists reserved
   alignas(128) uint32_t hub_cursor[2];  // next slice ticket
-  alignas(128) uint32_t units_done[2];  // warps that finished their own vertices
+  alignas(128) uint32_t units_done[2];  // CTAs whose warps have all finished their own vertices
 };
 
 // One command as the emulated device served it (times from %globaltimer, ns).
@@ -177,6 +177,10 @@ struct CtaState {
   uint32_t bar_count, bar_gen;       // grid barrier: arrivals in this CTA, generation
   uint32_t active;                   // application warps of this CTA that take part
   uint32_t ctas_active;              // CTAs with such warps
+  // slice queue (BFS, SpMV): warps of this CTA done with their own rows, and what the
+  // CTA's watching warp has seen of the queue (end_seen: phase + 1 once every warp of the
+  // grid is done and `end_count` slices are all there will be)
+  uint32_t own_done, watched, end_seen, end_count;
 };
 __device__ __forceinline__ CtaState &cta_state() {
   __shared__ CtaState cs;
@@ -2034,6 +2038,36 @@ static __device__ bool app_barrier(const Dev &d, uint32_t n_app, uint64_t deadli
 }
 
 
+// Slice queue of long rows (BFS: one per level parity, SpMV: 0).  own_work_done: this warp
+// queues no more slices (counted per CTA; lane 0).  slices_end: whether the queue is known to end at or before
+// ticket k (lane 0; `phase`: the level).  One warp of a CTA watches the shared counters for
+// the others, which look at shared memory: 2,000 warps polling one line would keep it from
+// the warps that still work, and polling seldom costs every level several microseconds.
+static __device__ __forceinline__ void own_work_done(const Dev &d, uint32_t par) {
+  CtaState &cs = cta_state();
+  fence_ar();
+  if (atomicAdd(&cs.own_done, 1u) + 1 == cs.active) {
+    cs.own_done = 0;
+    fence_ar();
+    atomicAdd(&d.run->units_done[par], 1u);
+  }
+}
+static __device__ __forceinline__ bool slices_end(const Dev &d, uint32_t par, uint32_t phase, uint32_t k) {
+  CtaState &cs = cta_state();
+  volatile uint32_t *seen = &cs.end_seen, *count = &cs.end_count;
+  if (*seen != phase + 1 && atomicCAS(&cs.watched, 0u, 1u) == 0u) {
+    if (ld_acq32(&d.run->units_done[par]) >= cs.ctas_active) {
+      *count = ld_acq32(&d.run->hub_count[par]);
+      __threadfence_block();
+      *seen = phase + 1;
+    }
+    atomicExch(&cs.watched, 0u);
+  }
+  if (*seen != phase + 1) return false;
+  __threadfence_block();
+  return *count <= k;
+}
+
 // Occupancy the engine is compiled for, in groups of kWarps warps per SM (register
 // budget): App::kMinBlocks if the application asks for more, else 2
 template <class App, class = void>
@@ -2094,7 +2128,7 @@ __global__ void __launch_bounds__(EngineShape<App>::threads, 1)
   for (uint32_t i = threadIdx.x; i < sizeof(Dev) / 4; i += EngineShape<App>::threads)
     ((uint32_t *)&cs.dev)[i] = ((const uint32_t *)&d)[i];
   if (threadIdx.x == 0) {
-    cs.done = cs.bar_count = cs.bar_gen = 0;
+    cs.done = cs.bar_count = cs.bar_gen = cs.own_done = cs.watched = cs.end_seen = cs.end_count = 0;
     cs.active = n_active > app_cta ? (n_active - app_cta + r.app_ctas - 1) / r.app_ctas : 0;
     cs.ctas_active = n_active < r.app_ctas ? n_active : r.app_ctas;
   }
