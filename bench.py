@@ -311,7 +311,7 @@ def run_bfs(args, torch, ag, dev, rank, world):
     edges = torch.zeros(1, dtype=torch.int64, device=dev)
     h_level = torch.empty(n, dtype=torch.int32, pin_memory=True)
     h_edges = torch.empty(1, dtype=torch.int64, pin_memory=True)
-    ctas, _ = ag.agile_launch_shape(ctx)
+    ctas, threads = ag.agile_launch_shape(ctx)
 
     def one(src, mode, e2e=False):
         ag.agile_invalidate(ctx, stream)
@@ -387,7 +387,7 @@ def run_bfs(args, torch, ag, dev, rank, world):
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": "int32", "data": "synthetic",
         "config": bfs_config(n, cols, srcs, cache_bytes, ways, cfg.num_queues, cfg.queue_depth),
-        "launch": {"ctas": ctas, "threads_per_cta": 256, "parallelism": f"replicas x{world}"},
+        "launch": {"ctas": ctas, "threads_per_cta": threads, "parallelism": f"replicas x{world}"},
         "sync": {"value": work_sync / (ms_sync * 1e-3), "unit": "edges/s", "ms_per_step": ms_sync / args.steps},
         "async_over_sync": ms_sync / ms_async,
         "roofline": {"bound": "host_link", "achieved": achieved, "peak": link_peak, "unit": "GB/s",

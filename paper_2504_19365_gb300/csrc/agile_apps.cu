@@ -1767,8 +1767,8 @@ int agile_embedding_bag(agile_ctx *c, uint64_t table_byte0, uint32_t rows, uint3
     return launch_engine(c, app, stream, warps, false);
   };
   if (dim <= 128) {
-    // three CTAs per SM (fewer registers a thread, so slower service warps) pay off only
-    // when the cache holds enough lines for more warps than two CTAs per SM give
+    // 24 warps an SM (80 registers a thread, so a slower miss path) pay off only when the
+    // cache holds enough lines for more warps than 16 an SM give
     uint64_t want = c->cfg.app_warps ? c->cfg.app_warps : warps;
     if (want > app_warps_of_grid<EmbApp<1, 2>>(c)) return go(EmbApp<1, 3>{});
     return go(EmbApp<1, 2>{});
