@@ -22,13 +22,15 @@ __device__ __forceinline__ bool page_ok(const Dev &d, uint64_t page) {
   return page < d.store_bytes / kPage;
 }
 
-// asyncRead / prefetch (Sec. 3.1, Listing 1 Methods 1 and 2).  Each app warp takes 32
+// asyncRead / prefetch (Sec. 3.1, Listing 1 Methods 1 and 2).  Each app warp takes up to 32
 // requests at a time.  prefetch_only: issue the misses and return.  Otherwise every
 // page is copied line -> d_dst with the line pinned for the copy only.  SYNC requests
-// each page and waits for it before requesting the next.  ASYNC keeps the requests of two
-// halves of 16 in flight: one half is requested before the half in front of it is copied, so
-// that the device works while the warp copies (bound: the host link; 65,536 pages of which
-// 60 k miss took 1.56 ms with 32 requested, waited for and copied in turn).
+// each page and waits for it before requesting the next.  ASYNC requests kPart pages
+// before it copies the kPart in front of them, so that the device works while the warp
+// copies.  Many warps with few pages in flight each, because a warp copies in order and a deep
+// queue makes it wait for its next page: 65,536 random pages of which 60 k miss take
+// 1.31 ms with parts of 2, 1.42 of 4, 1.44 of 8 and 1.57 of 16 (bound: the host link,
+// 1.16 ms); 8,192 pages through 4,096 lines 0.27, 0.28, 0.40 and 0.54 ms.
 struct ReadApp {
   const uint64_t *pages;
   uint32_t n;
@@ -38,10 +40,11 @@ struct ReadApp {
   // no request ahead of need: the launch uses every queue pair for demand
   bool demand_only() const { return !prefetch_only; }  // reads are waited for in both modes
   int prefetch_only;
+  static constexpr uint32_t kPart = 2;  // requests asked for together (ASYNC)
 
   // page of request i (want: there is one, inside the store)
-  __device__ __forceinline__ uint64_t request(const Dev &d, uint64_t i, bool &want) const {
-    want = i < n;
+  __device__ __forceinline__ uint64_t request(const Dev &d, uint64_t i, bool mine, bool &want) const {
+    want = mine && i < n;
     uint64_t page = want ? pages[i] : 0;
     if (want && !page_ok(d, page)) {
       set_error(d, AGILE_EINVAL);
@@ -98,38 +101,43 @@ struct ReadApp {
 
   __device__ void run(const Dev &d, const AppCtx &a) const {
     unsigned l = lane_id();
-    const uint64_t stride = (uint64_t)a.n_warps * 32;
-    uint64_t base = (uint64_t)a.warp * 32;
+    // requests a warp takes at a time: up to 32, fewer when that leaves warps without any
+    const uint32_t each = (n + a.n_warps - 1) / a.n_warps;
+    const uint32_t take = min(32u, (each + kPart - 1) / kPart * kPart);
+    const uint64_t stride = (uint64_t)a.n_warps * take;
+    uint64_t base = (uint64_t)a.warp * take;
     bool want = false;
-    uint64_t page = base < n ? request(d, base + l, want) : 0;
+    uint64_t page = base < n ? request(d, base + l, l < take, want) : 0;
     uint64_t t = AGILE_TOKEN_HIT;  // of the page at hand; its first half is requested one step early
     const bool async = mode == AGILE_ASYNC && !prefetch_only;
-    auto ask = [&](uint64_t pg, bool w, bool half, uint64_t &token) {
+    auto ask = [&](uint64_t pg, bool w, uint32_t part, uint64_t &token) {
       uint64_t got = AGILE_TOKEN_HIT;
-      w = w && (l >= 16) == half;
+      w = w && l / kPart == part;
       if (__any_sync(kFull, w) && !warp_request(d, w, pg, a.q0, false, a.deadline, &got)) return false;
       if (w) token = got;
       return true;
     };
-    if (async && !ask(page, want, false, t)) return;
+    if (async && !ask(page, want, 0, t)) return;
     for (; base < n; base += stride) {
       if (aborted(d)) return;
       if (prefetch_only) {
         stat_warp(d, S_PREFETCHES, want ? 1u : 0u);
         if (!warp_request(d, want, page, a.q0, false, a.deadline, nullptr, nullptr, nullptr, true)) return;
-        page = base + stride < n ? request(d, base + stride + l, want) : 0;
+        want = false;
+        page = base + stride < n ? request(d, base + stride + l, l < take, want) : 0;
         continue;
       }
       unsigned grp = __match_any_sync(kFull, want ? page : ~0ull);
       const unsigned all = __ballot_sync(kFull, want);
       bool want2 = false;
       uint64_t page2 = 0, t2 = AGILE_TOKEN_HIT;
-      if (base + stride < n) page2 = request(d, base + stride + l, want2);
+      if (base + stride < n) page2 = request(d, base + stride + l, l < take, want2);
       if (async) {
-        if (!ask(page, want, true, t)) return;
-        if (!copy(d, a, base, page, all & 0xFFFFu)) return;
-        if (!ask(page2, want2, false, t2)) return;
-        if (!copy(d, a, base, page, all & 0xFFFF0000u)) return;
+        for (uint32_t part = 0; part < take / kPart; ++part) {
+          const bool last = part + 1 == take / kPart;
+          if (last ? !ask(page2, want2, 0, t2) : !ask(page, want, part + 1, t)) return;
+          if (!copy(d, a, base, page, all & (((1u << kPart) - 1) << (kPart * part)))) return;
+        }
       } else {
         for (unsigned m = all; m; m &= m - 1) {
           const int j = __ffs(m) - 1;
@@ -719,7 +727,7 @@ int agile_read_async(agile_ctx *c, const uint64_t *d_pages, uint32_t n, void *d_
   if (((uintptr_t)d_dst) & 15) return AGILE_EINVAL;
   if (n == 0) return AGILE_OK;
   ReadApp app{d_pages, n, (uint8_t *)d_dst, d_tok, mode, 0};
-  return launch_engine(c, app, stream, warps_for_cache(c, mode == AGILE_ASYNC ? 48 : 4, 8));
+  return launch_engine(c, app, stream, warps_for_cache(c, mode == AGILE_ASYNC ? 3 * ReadApp::kPart : 4, 8));
 }
 
 int agile_prefetch(agile_ctx *c, const uint64_t *d_pages, uint32_t n, void *stream) {
