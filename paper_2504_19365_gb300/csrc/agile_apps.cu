@@ -123,6 +123,7 @@ struct EmbApp {
     int pr = P_HIT;
     p.line = 0;
     if (p.leader) pr = cache_probe(d, p.pg, true, p.line);
+    __syncwarp();  // the pins' acquires come before every lane's reads of the lines
     p.ok = __all_sync(kFull, !p.leader || pr == P_HIT);
     if (p.ok) {  // counted here; a bag that is not all resident is counted by gather_sum
       stat_warp(d, S_WARP_COALESCED, (want && !p.leader) ? 1u : 0u);

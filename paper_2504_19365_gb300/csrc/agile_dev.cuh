@@ -1088,7 +1088,9 @@ static __device__ __noinline__ Requested warp_request_body(bool want, uint64_t p
       }
       __syncwarp();
       if (m == M_ISSUED) m = cache_reserve(d, page, q0, c, pf);
-      // MODIFIED victims are copied to their staging pages by the whole warp
+      // MODIFIED victims are copied to their staging pages by the whole warp: its reads come
+      // after the claiming lane's fence (votes and shuffles order no memory)
+      __syncwarp();
       for (unsigned wb = __ballot_sync(kFull, m == M_ISSUED && c.wb); wb; wb &= wb - 1) {
         const int j = __ffs(wb) - 1;
         const uint64_t src = __shfl_sync(kFull, (uint64_t)line_ptr(d, c.line), j);
@@ -1173,6 +1175,7 @@ __device__ __forceinline__ int warp_probe_pin(const Dev &d, uint64_t page, uint3
       }
     }
   }
+  __syncwarp();  // the pin's acquire comes before every lane's reads of the line
   return __shfl_sync(kFull, pr, w);
 }
 
@@ -1474,6 +1477,7 @@ static __device__ bool gather_sum(const Dev &d, const AppCtx &a, uint32_t begin,
         got = tag_page(old) == pg && (ost == ST_READY || ost == ST_MODIFIED);
         if (!got) cache_unpin(d, line);  // evicted since the probe
       }
+      __syncwarp();  // the pins' acquires come before every lane's reads of the lines
       const unsigned lost = __ballot_sync(kFull, mine && !got);
       uint32_t myline = __shfl_sync(kFull, line, lead_lane & 31);
       if (lost) {

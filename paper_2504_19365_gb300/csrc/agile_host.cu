@@ -61,6 +61,7 @@ struct ReadApp {
     while (todo) {
       uint32_t line = 0;
       const bool hit = ((todo >> l) & 1u) && cache_probe(d, page, true, line) == P_HIT;
+      __syncwarp();  // the pins' acquires come before every lane's reads of the lines
       const unsigned got = __ballot_sync(kFull, hit);
       for (unsigned m = got; m;) {
         const int j = __ffs(m) - 1;
@@ -223,6 +224,7 @@ struct WriteApp {
         backoff(ns);
       }
       line = __shfl_sync(kFull, line, 0);
+      __syncwarp();  // lane 0 owns the line, and its copy of a MODIFIED victim is done
       // 3. new contents into the line; publish it READY (a full page supersedes it)
       warp_copy_page(line_ptr(d, line), src + i * kPage);
       __threadfence();
