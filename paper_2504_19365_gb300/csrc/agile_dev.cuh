@@ -355,16 +355,23 @@ __device__ __forceinline__ void lane_copy_page(void *dst, const void *src) {
 // Alg. 2, check_full: reserve n consecutive slots of queue q.  A slot is free when
 // the command that used it last has completed (state EMPTY) and fewer than depth-1
 // commands are outstanding (the NVMe full rule).  Never waits.
-// `w`: the queue's reservation word as read before.
+// `w`: the queue's reservation word as read before.  Another command may have taken the
+// slot it names since, so the queue is full only if the word has not changed.
 __device__ __forceinline__ bool sq_try_reserve(const Dev &d, uint32_t q, uint32_t n, uint64_t w,
                                                uint32_t &slot, uint32_t &ticket) {
   unsigned long long *rp = &d.sq_resv[q];
   for (int tries = 0; tries < 4; ++tries) {
     uint32_t t = (uint32_t)w, infl = (uint32_t)(w >> 32);
-    if (infl + n > d.depth - 1) return false;
-    for (uint32_t k = 0; k < n; ++k) {
+    bool room = infl + n <= d.depth - 1;
+    for (uint32_t k = 0; k < n && room; ++k) {
       uint64_t st = ld_acq64(&d.sqe_state[(uint64_t)q * d.depth + ((t + k) & d.dmask)]);
-      if ((st & 3) != SQE_EMPTY) return false;
+      room = (st & 3) == SQE_EMPTY;
+    }
+    if (!room) {
+      const uint64_t now = ld_rlx64(rp);
+      if (now == w) return false;
+      w = now;
+      continue;
     }
     uint64_t nw = ((uint64_t)(infl + n) << 32) | (uint32_t)(t + n);
     uint64_t old = atomicCAS(rp, (unsigned long long)w, (unsigned long long)nw);
