@@ -1458,7 +1458,10 @@ static __device__ bool gather_sum(const Dev &d, const AppCtx &a, uint32_t begin,
     uint32_t line = 0;
     int pr = P_HIT;
     if (leader) pr = cache_probe(d, pg, false, line);
-    if (first) stat_warp(d, S_HITS, (leader && pr == P_HIT) ? 1u : 0u);
+    if (first) {
+      stat_warp(d, S_HITS, (leader && pr == P_HIT) ? 1u : 0u);
+      stat_warp(d, S_BUSY_HITS, (leader && pr == P_BUSY) ? 1u : 0u);
+    }
     first = false;
     const unsigned away = __ballot_sync(kFull, leader && pr != P_HIT);
     const bool ask = leader && pr == P_MISS && (uint32_t)__popc(away & ((1u << l) - 1)) < window;
