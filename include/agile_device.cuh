@@ -37,7 +37,10 @@
  *       out or the arguments are out of range (AGILE_EINVAL, reported by agile_check).
  *
  * a.warp / a.n_warps give the warp's index among the application warps; a.deadline is
- * the launch's own bound (cfg.wait_timeout_ns after the start).
+ * the launch's own bound (cfg.wait_timeout_ns after the start).  A CTA has agile::kWarps
+ * warps (agile::kThreads threads): shared memory that run() keeps for each warp of its CTA is
+ * sized by kWarps and indexed by threadIdx.x / 32.  The launch keeps sizeof(agile::CtaState)
+ * bytes of the CTA's static shared memory for itself.
  *
  * Host side:  int rc = agile::launch_user(ctx, app, stream, app_warps);
  *   launches `app` on `stream` over the context's queues and cache (all of the grid's
@@ -111,21 +114,18 @@ int launch_user(agile_ctx *ctx, const App &app, void *stream, uint32_t app_warps
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return AGILE_ECUDA;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return AGILE_ECUDA;
-  if (engine_shared<App>() > 0 &&
-      cudaFuncSetAttribute(engine_kernel<App>, cudaFuncAttributeMaxDynamicSharedMemorySize, engine_shared<App>()) !=
-          cudaSuccess)
-    return AGILE_ECUDA;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, engine_kernel<App>, EngineShape<App>::threads,
-                                                    engine_shared<App>()) != cudaSuccess ||
+  using Engine = UserApp<App>;
+  static_assert(EngineShape<Engine>::threads == kThreads, "a user kernel's CTA has kWarps warps");
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, engine_kernel<Engine>, kThreads, 0) != cudaSuccess ||
       per_sm <= 0)
     return AGILE_ECUDA;
   d.app_active = app_warps;
   r = agile_run_reset(ctx, stream);
   if (r) return r;
-  App a = app;
+  Engine a{app};
   void *args[] = {(void *)&d, (void *)&a};
-  if (cudaLaunchCooperativeKernel((const void *)engine_kernel<App>, dim3(per_sm * sms),
-                                  dim3(EngineShape<App>::threads), args, engine_shared<App>(), (cudaStream_t)stream) != cudaSuccess)
+  if (cudaLaunchCooperativeKernel((const void *)engine_kernel<Engine>, dim3(per_sm * sms), dim3(kThreads), args, 0,
+                                  (cudaStream_t)stream) != cudaSuccess)
     return AGILE_ECUDA;
   return AGILE_OK;
 }

@@ -24,9 +24,11 @@
 namespace agile {
 
 constexpr uint32_t kPage = 4096;
-// An engine CTA fills its SM: kWarps warps times the occupancy its application is compiled
-// for (MinBlocks, 2 by default: 16 warps of 128 registers).
+// A CTA of a user kernel (agile::launch_user) has kWarps warps, as many CTAs on an SM as its
+// application is compiled for (MinBlocks, 2 by default: 16 warps of 128 registers an SM).
+// A library call's engine has the same warps in one CTA.
 constexpr int kWarps = 8;
+constexpr int kThreads = kWarps * 32;
 constexpr unsigned kFull = 0xffffffffu;
 
 // ---------------------------------------------------------------- tag word (Sec. 3.4)
@@ -2092,10 +2094,28 @@ template <class App>
 struct MinBlocks<App, decltype((void)App::kMinBlocks, void())> {
   static constexpr int value = App::kMinBlocks;
 };
+// CTAs that share an SM: one, which has all of its warps, unless the application asks for more
+template <class App, class = void>
+struct CtasPerSm {
+  static constexpr int value = 1;
+};
+template <class App>
+struct CtasPerSm<App, decltype((void)App::kCtasPerSm, void())> {
+  static constexpr int value = App::kCtasPerSm;
+};
 template <class App>
 struct EngineShape {
-  static constexpr int warps = kWarps * MinBlocks<App>::value;
+  static constexpr int ctas = CtasPerSm<App>::value;
+  static constexpr int warps = kWarps * MinBlocks<App>::value / ctas;
   static constexpr int threads = warps * 32;
+};
+// A user's application: its CTAs have kWarps warps, so that what it keeps for each warp of
+// a CTA is sized by kWarps.  Of its members only run() and kMinBlocks mean anything here.
+template <class App>
+struct UserApp {
+  static constexpr int kMinBlocks = MinBlocks<App>::value, kCtasPerSm = kMinBlocks;
+  App app;
+  __device__ __forceinline__ void run(const Dev &d, const AppCtx &a) const { app.run(d, a); }
 };
 // dynamic shared memory an application wants for each warp of the CTA
 template <class App, class = void>
@@ -2124,7 +2144,7 @@ struct HasIdle<App, decltype((void)&App::idle)> {
 };
 
 template <class App>
-__global__ void __launch_bounds__(EngineShape<App>::threads, 1)
+__global__ void __launch_bounds__(EngineShape<App>::threads, EngineShape<App>::ctas)
     engine_kernel(const __grid_constant__ Dev d, const __grid_constant__ App app) {
   if constexpr (HasIdle<App>::value) {
     if (app.idle(d)) return;
