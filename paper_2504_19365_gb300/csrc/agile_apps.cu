@@ -448,7 +448,6 @@ struct BfsAppT {
   const uint8_t *h_off = nullptr, *h_col = nullptr;  // kDirect: the CSR arrays in HBM
 
   static constexpr uint32_t kChunk = 128;
-  static constexpr uint32_t kBigShare = 5;  // eighths of a dense level claimed kChunk at a time
 
   __device__ __forceinline__ uint64_t tag(const Dev &d, int32_t L) const {
     return (launch_epoch(d) << 32) | (uint32_t)(L + 1);
@@ -812,25 +811,18 @@ struct BfsAppT {
       uint32_t found = 0;
       Pin pc{0, 0, false};
       bool ok = true;
-      // the last part of a dense level is claimed in units of 32: a chunk of 128 takes a
-      // fifth of the level, and whoever claims one last would hold the others up
-      const uint32_t big = frontier * 256 < n ? wide : csize;
-      const uint32_t n_big = big == kChunk && csize == kChunk ? n / kChunk * kBigShare / 8 : (uint32_t)(((uint64_t)n + big - 1) / big);
-      const uint64_t small0 = (uint64_t)n_big * big;
-      const uint32_t nchunks = n_big + (small0 < n ? (uint32_t)((n - small0 + 31) / 32) : 0u);
-      uint32_t c = 0, at = 0, span = 0, step = 32;  // the claimed chunk and how far the warp is in it
+      const uint32_t span = frontier * 256 < n ? wide : csize, step = min(span, kChunk), U = step / 32;
+      const uint32_t nchunks = (uint32_t)(((uint64_t)n + span - 1) / span);
+      uint32_t c = 0, at = span;  // the claimed chunk and how far the warp is in it
       for (; ok; at += step) {
         if (at >= span) {
           if (l == 0) c = atomicAdd(&d.run->work[L & 1], 1u);
           c = __shfl_sync(kFull, c, 0);
           if (c >= nchunks || aborted(d)) break;
           at = 0;
-          span = c < n_big ? big : 32;
-          step = min(span, kChunk);
         }
-        const uint64_t v00 = (c < n_big ? (uint64_t)c * big : small0 + (uint64_t)(c - n_big) * 32) + at;
+        const uint64_t v00 = (uint64_t)c * span + at;
         if (v00 >= n) continue;
-        const uint32_t U = step / 32;
         const uint32_t c0 = (uint32_t)v00;
         // the chunk's level words, all in flight together: bit k of fbits says whether
         // the lane's vertex of unit k is in the frontier (a word equal to L was written
