@@ -30,7 +30,8 @@ struct EmbApp {
   // no request ahead of need: the launch uses every queue pair for demand
   bool demand_only() const { return mode == AGILE_SYNC; }
   uint32_t ahead;  // rows requested ahead of the one being summed (ASYNC), 1..32
-  uint32_t group;  // pages requested and not yet used, at most (cache-sized), 1..32
+  uint32_t group;  // rows of a bag that is pinned as a whole, hints of a round, at most (cache-sized), 1..32
+  uint32_t window;  // pages a gather has requested and not yet used, at most, 1..32
   // bags left by the resident pass: positions 0 .. run->pending - 1 name bags list[pos];
   // n_bags bounds the positions
   const uint32_t *list;
@@ -167,7 +168,7 @@ struct EmbApp {
       // keep the pages of the next `ahead` rows of the stream requested
       if (async && !issue_rows(d, a, pf, cnt, bo)) return false;
       bool missed = false;
-      if (!gather_sum<MF4>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, group, &missed))
+      if (!gather_sum<MF4>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, window, &missed))
         return false;
       if (missed) bo.missed();
     }
@@ -281,7 +282,8 @@ struct PipeApp {
   uint32_t mode;
   // no request ahead of need: the launch uses every queue pair for demand
   bool demand_only() const { return mode == AGILE_SYNC; }
-  uint32_t group;     // pages requested and not yet used, at most (cache-sized), 1..32
+  uint32_t group;     // hints of a round, at most (cache-sized), 1..32
+  uint32_t window;    // pages a gather has requested and not yet used, at most, 1..32
   uint32_t ahead;     // async: rows of the warp's row stream requested ahead (cache-sized)
 
   __device__ __forceinline__ uint64_t row_page(uint32_t k, uint64_t r) const {
@@ -354,7 +356,7 @@ struct PipeApp {
           uint64_t byte = (uint64_t)k * tstride + r * dim * 4;
           if (async && !issue_ahead(d, a, pf, cnt, units, bo)) return;
           bool missed = false;
-          if (!gather_sum<MF4>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, group, &missed))
+          if (!gather_sum<MF4>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, window, &missed))
             return;
           if (missed) bo.missed();
         }
@@ -1578,13 +1580,6 @@ __global__ void bfs_init_kernel(int32_t *level, uint32_t *vis, uint32_t n, int32
   if (i < (n + 31ull) / 32) vis[i] = (i == (uint64_t)src / 32) ? 1u << (src % 32) : 0u;
 }
 
-// pages a warp requests before it uses them: with `warps` warps each holding that many
-// lines at once, at most half of the cache is waited for
-uint32_t pin_group(const agile_ctx *c, uint32_t warps) {
-  uint64_t g = c->dev.nlines / (2ull * std::max<uint32_t>(1, warps));
-  return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(32, g));
-}
-
 int bfs_check(agile_ctx *c, uint64_t offsets_byte0, uint64_t cols_byte0, uint32_t n_vertices, int32_t src,
               int32_t *d_level, uint32_t mode) {
   if (!c || mode > 1 || !d_level) return AGILE_EINVAL;
@@ -1756,7 +1751,7 @@ int agile_embedding_bag(agile_ctx *c, uint64_t table_byte0, uint32_t rows, uint3
     uint64_t ahead = look ? c->dev.nlines / (2ull * run) : 0;
     ahead = std::max<uint64_t>(1, std::min<uint64_t>(32, ahead * c->cfg.prefetch_depth));
     App app{table_byte0 / kPage, rows, dim, d_idx, d_offsets, n_bags, d_out, look ? mode : (uint32_t)AGILE_SYNC,
-            (uint32_t)ahead, pin_group(c, run), list};
+            (uint32_t)ahead, pin_group(c, run), gather_window(c, run), list};
     return launch_engine(c, app, stream, warps, false);
   };
   if (dim <= 128) {
@@ -1802,7 +1797,8 @@ int agile_embedding_pipeline(agile_ctx *c, uint64_t table_byte0, uint64_t table_
     uint64_t ahead = look ? c->dev.nlines / (2ull * run) * c->cfg.prefetch_depth : 0;
     ahead = std::max<uint64_t>(1, std::min<uint64_t>(per_unit, ahead));
     App app{table_byte0 / kPage, table_stride, n_tables, rows, dim, d_idx, pooling, n_bags, n_batches,
-            compute_iters, d_out, look ? mode : (uint32_t)AGILE_SYNC, group, (uint32_t)ahead};
+            compute_iters, d_out, look ? mode : (uint32_t)AGILE_SYNC, group, gather_window(c, run),
+            (uint32_t)ahead};
     return launch_engine(c, app, stream, warps);
   };
   if (dim <= 128) return go(PipeApp<1>{});

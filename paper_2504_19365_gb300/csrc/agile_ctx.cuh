@@ -51,6 +51,23 @@ inline uint32_t warps_for_cache(const agile_ctx *c, uint64_t pages_per_warp, uin
   return (uint32_t)std::max<uint64_t>(floor_warps, w);
 }
 
+// Pages a warp requests before it uses them: with `warps` warps each holding that many
+// lines at once, at most half of the cache is waited for.
+inline uint32_t pin_group(const agile_ctx *c, uint32_t warps) {
+  uint64_t g = c->dev.nlines / (2ull * std::max<uint32_t>(1, warps));
+  return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(32, g));
+}
+// ... and, for a gather, the windows of all warps together take the queue slots there are:
+// thousands of lanes that claim lines and find no slot for their reads keep the words of
+// queues and sets busy.  2,048 warps with windows of 32 on 128 x 255 slots: 8 M uniform
+// lookups took 22.3 ms, 17.9 with windows of 15; on 32 x 63 slots 1/2 M took 12.0 ms, 5.0
+// with windows of 1.  Up to 1,024 requests (32 warps with windows of 32) are let wait on
+// any queues: they keep few and short queues full (2 x 63 slots: 75 ms, 87 with windows of 3).
+inline uint32_t gather_window(const agile_ctx *c, uint32_t warps) {
+  uint64_t s = std::max<uint64_t>((uint64_t)c->dev.Q * (c->dev.depth - 1), 1024) / std::max<uint32_t>(1, warps);
+  return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(pin_group(c, warps), s));
+}
+
 // Largest co-resident grid for this engine instantiation (cooperative launch rule:
 // every CTA must be resident at once, because the service warps and the waiting app
 // warps of one launch depend on each other).

@@ -89,7 +89,7 @@ struct ServeApp {
   uint32_t mode;
   // serving requests only what it sums: every queue pair carries demand
   bool demand_only() const { return true; }
-  uint32_t group;
+  uint32_t window;  // pages a gather has requested and not yet used, at most
 
   __device__ void schedule(const Dev &d, const AppCtx &a) const {
     // lane 0 only
@@ -160,7 +160,7 @@ struct ServeApp {
       uint64_t byte = r * dim * 4;
       if (mode == AGILE_ASYNC && !warp_request(d, l < cnt, page0 + byte / kPage, a.q0, false, a.deadline))
         return false;
-      if (!gather_sum<1>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, group)) return false;
+      if (!gather_sum<1>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, window)) return false;
     }
     if (l < nf4) ((float4 *)(out + (uint64_t)b * dim))[l] = acc[0];
     return true;
@@ -277,11 +277,11 @@ int agile_serve_start(agile_ctx *c, uint32_t ring_slots, uint32_t mode, uint64_t
   AGILE_CUDA_TRY(cudaHostGetDevicePointer(&done_d, s->done, 0));
   AGILE_CUDA_TRY(cudaHostGetDevicePointer(&stop_d, s->stop, 0));
   uint32_t warps = warps_for_cache(c, 4, 32);
-  // pin groups sized by the warps that run (one of them schedules)
+  // windows sized by the warps that run (one of them schedules)
   uint32_t run = running_app_warps<ServeApp>(c, warps + 1);
   ServeApp app{(ServeSlot *)ring_d, (unsigned long long *)done_d, (const uint32_t *)stop_d,
                (ServeDev *)s->dstate, (ReqState *)((ServeDev *)s->dstate + 1), ring_slots,
-               c->dev.nlines / 2, mode, std::max<uint32_t>(1, std::min<uint32_t>(32, (uint32_t)(c->dev.nlines / (2ull * run))))};
+               c->dev.nlines / 2, mode, gather_window(c, run)};
   uint64_t saved = c->dev.session_ns;
   c->dev.session_ns = session_ns ? session_ns : 60ull * 1000 * 1000 * 1000;
   int r = launch_engine(c, app, stream, warps + 1);
