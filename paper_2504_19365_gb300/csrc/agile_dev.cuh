@@ -1286,6 +1286,13 @@ struct AppCtx {
   uint64_t deadline;
 };
 
+// Requests a warp takes at a time when `warps` warps share `n`: enough for all of them, a
+// multiple of `part`, at most 32.
+__host__ __device__ constexpr uint32_t requests_a_step(uint64_t n, uint32_t warps, uint32_t part) {
+  const uint64_t each = (n + warps - 1) / warps, parts = (each + part - 1) / part;
+  return parts < 32 / part ? (uint32_t)parts * part : 32 / part * part;
+}
+
 // ================================================================ user kernel API
 // The device side of Listing 1 (Sec. 3.5) for kernels that run inside a library launch
 // (agile_device.cuh launches them): a warp's lanes issue reads, continue with other

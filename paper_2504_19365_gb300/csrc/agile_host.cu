@@ -103,8 +103,7 @@ struct ReadApp {
   __device__ void run(const Dev &d, const AppCtx &a) const {
     unsigned l = lane_id();
     // requests a warp takes at a time: up to 32, fewer when that leaves warps without any
-    const uint32_t each = (n + a.n_warps - 1) / a.n_warps;
-    const uint32_t take = min(32u, (each + kPart - 1) / kPart * kPart);
+    const uint32_t take = requests_a_step(n, a.n_warps, kPart);
     const uint64_t stride = (uint64_t)a.n_warps * take;
     uint64_t base = (uint64_t)a.warp * take;
     bool want = false;
