@@ -73,13 +73,16 @@ inline uint32_t gather_window(const agile_ctx *c, uint32_t warps) {
 // warps of one launch depend on each other).
 template <class App>
 int engine_grid(agile_ctx *c) {
+  // the allowance for dynamic shared memory is a property of the kernel on the current
+  // device: set for every launch, so that a context on a second device has it too
+  if (engine_shared<App>() > 0 &&
+      (cudaSetDevice(c->device) != cudaSuccess ||
+       cudaFuncSetAttribute(engine_kernel<App>, cudaFuncAttributeMaxDynamicSharedMemorySize, engine_shared<App>()) !=
+           cudaSuccess))
+    return 0;
   static int per_sm = -1;  // one value per instantiation
   if (per_sm < 0) {
     int n = 0;
-    if (engine_shared<App>() > 0 &&
-        cudaFuncSetAttribute(engine_kernel<App>, cudaFuncAttributeMaxDynamicSharedMemorySize, engine_shared<App>()) !=
-            cudaSuccess)
-      return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, engine_kernel<App>, EngineShape<App>::threads,
                                                       engine_shared<App>()) != cudaSuccess)
       return 0;
