@@ -582,6 +582,24 @@ def check_or_raise(ag, ctx):
         raise RuntimeError(f"device error: {ag.strerror(err)}")
 
 
+def compute_round_ms(time_ms, first=2000):
+    """Cost of one round of the pipeline's compute phase, from time_ms(rounds), the time of a
+    call with that many rounds on a warm cache.  Misses (a cache too small to be warm) hide
+    compute, so that the difference to the call without compute says nothing while it is
+    small: the rounds are doubled until the call takes three times as long as the one
+    without, and the next doubling is all compute.  No call here takes more than about
+    twelve times the one without compute."""
+    t0 = time_ms(0)
+    n, tn = first, time_ms(first)
+    while n < 1 << 30:
+        t2 = time_ms(2 * n) if tn >= 3 * t0 + 0.2 else 0.0
+        if t2 > tn:
+            return (t2 - tn) / n
+        n *= 2
+        tn = t2 or time_ms(n)
+    raise RuntimeError("the compute phase cannot be calibrated")
+
+
 def overlap_sweep(torch, ag, dev, ctx, stride, nt, rows, dim, nbags, pool, stream, flush, batches_full=4, reps=5):
     """Config-3 overlap sweep on an open context: per batch the lookups of nt tables x
     nbags bags x pooling, then the FP32 compute phase sized to r x the sync I/O time
@@ -610,8 +628,8 @@ def overlap_sweep(torch, ag, dev, ctx, stride, nt, rows, dim, nbags, pool, strea
         # compute cost per iteration on a warm cache (this batch set fits in it)
         go(ag.AGILE_SYNC, 0, cold=False)
         w0 = statistics.median(go(ag.AGILE_SYNC, 0, cold=False) for _ in range(3))
-        w1 = statistics.median(go(ag.AGILE_SYNC, 2000, cold=False) for _ in range(3))
-        per_iter = max(1e-6, (w1 - w0) / 2000)
+        per_iter = compute_round_ms(
+            lambda k: statistics.median(go(ag.AGILE_SYNC, k, cold=False) for _ in range(3)))
         pts = []
         for r in (0.25, 0.5, 1, 2, 4, 8):
             iters = max(1, int(r * t_io / per_iter))
@@ -711,41 +729,44 @@ def run_sweeps(args, torch, ag, dev):
                     mode, stream))
             go(ag.AGILE_SYNC, 0)
             t_io = go(ag.AGILE_SYNC, 0)
-            w0 = go(ag.AGILE_SYNC, 0, cold=False)
-            w1 = go(ag.AGILE_SYNC, 20000, cold=False)
-            # one round is a few dependent FMAs per element: at least 1 ns, whatever the
-            # calibration noise
-            per_iter = max(1e-6, (w1 - w0) / 20000)
+            go(ag.AGILE_SYNC, 0, cold=False)
+            per_iter = compute_round_ms(lambda k: go(ag.AGILE_SYNC, k, cold=False))
+            check_or_raise(ag, ctx)
             iters = max(1, int(t_io / per_iter))
             ts = go(ag.AGILE_SYNC, iters)
             ta = go(ag.AGILE_ASYNC, iters)
+            check_or_raise(ag, ctx)
             res[name] = {"sync_ms": round(ts, 3), "async_ms": round(ta, 3), "async_speedup": round(ts / ta, 3),
                          "iters": iters}
         ag.agile_config_parallelism(ctx, 0)
-        err = ag.agile_check(ctx)
-        if err:
-            raise RuntimeError(f"device error: {ag.strerror(err)}")
         return res
+
+    def point_or_error(*a):  # one point that fails does not take the others with it
+        try:
+            return point(*a)
+        except Exception as e:  # noqa: BLE001
+            ag.agile_config_parallelism(a[0], 0)
+            return {"error": f"{type(e).__name__}: {e}"}
 
     out = {"workload": "8 x 1,000,000 x 64 FP32 tables (2.05 GB), Zipf 1.05, pooling 32, compute at CTC 1, "
                        "cold cache per call"}
     ctx = context()
     try:
-        out["batch_size"] = {str(nb): point(ctx, nb, max(1, min(16, 2048 // nb))) for nb in (1, 16, 128, 1024, 2048)}
+        out["batch_size"] = {str(nb): point_or_error(ctx, nb, max(1, min(16, 2048 // nb))) for nb in (1, 16, 128, 1024, 2048)}
     finally:
         ag.agile_destroy(ctx)
     out["queue_pairs_depth_64"] = {}
     for q in (1, 2, 4, 8, 16):
         ctx = context(queues=q, depth=64)
         try:
-            out["queue_pairs_depth_64"][str(q)] = point(ctx, 2048, 1)
+            out["queue_pairs_depth_64"][str(q)] = point_or_error(ctx, 2048, 1)
         finally:
             ag.agile_destroy(ctx)
     out["cache_bytes"] = {}
     for cb in (1 << 20, 16 << 20, 256 << 20, 2 << 30):
         ctx = context(cache_bytes=cb)
         try:
-            out["cache_bytes"][f"{cb >> 20}MiB"] = point(ctx, 2048, 1)
+            out["cache_bytes"][f"{cb >> 20}MiB"] = point_or_error(ctx, 2048, 1)
         finally:
             ag.agile_destroy(ctx)
     return out
