@@ -190,7 +190,8 @@ AGILE_API int agile_store_read(agile_ctx *ctx, uint64_t off, void *host_dst, uin
 /* asyncRead (Sec. 3.1, Listing 1 Method-2): for i < n, copy store page d_pages[i]
  * through the cache into d_dst + i*4096 and write its token to d_tok[i] (may be
  * NULL).  d_pages: uint64 page numbers; d_dst: n*4096 bytes, 16-byte aligned.
- * mode AGILE_ASYNC issues all misses of a warp's pages before waiting for any. */
+ * mode AGILE_ASYNC requests a warp's next two pages before it copies the two in front of
+ * them; AGILE_SYNC requests each page and waits for it before it requests the next. */
 AGILE_API int agile_read_async(agile_ctx *ctx, const uint64_t *d_pages, uint32_t n, void *d_dst,
                      agile_token *d_tok, uint32_t mode, void *stream);
 

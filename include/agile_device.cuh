@@ -101,7 +101,7 @@ __device__ __forceinline__ int share_release(const Dev &d, const AppCtx &a, bool
   return agile::share_release(d, a, want, page);
 }
 // grid barrier over the launch's application warps (every one must call it)
-__device__ __forceinline__ bool barrier(const Dev &d, const AppCtx &a) { return app_barrier(d, a.n_warps, a.deadline); }
+__device__ __forceinline__ bool barrier(const Dev &d, const AppCtx &a) { return app_barrier(d, a.deadline); }
 
 }  // namespace dev
 

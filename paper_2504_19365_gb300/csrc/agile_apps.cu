@@ -168,7 +168,7 @@ struct EmbApp {
       // keep the pages of the next `ahead` rows of the stream requested
       if (async && !issue_rows(d, a, pf, cnt, bo)) return false;
       bool missed = false;
-      if (!gather_sum<MF4>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, window, &missed))
+      if (!gather_sum<MF4>(d, a, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, window, &missed))
         return false;
       if (missed) bo.missed();
     }
@@ -250,7 +250,6 @@ struct EmbApp {
       store_out(b, acc, nf4);
       cur = nxt;
     }
-    (void)l;
   }
 };
 
@@ -356,7 +355,7 @@ struct PipeApp {
           uint64_t byte = (uint64_t)k * tstride + r * dim * 4;
           if (async && !issue_ahead(d, a, pf, cnt, units, bo)) return;
           bool missed = false;
-          if (!gather_sum<MF4>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, window, &missed))
+          if (!gather_sum<MF4>(d, a, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, window, &missed))
             return;
           if (missed) bo.missed();
         }
@@ -382,11 +381,12 @@ struct PipeApp {
 
 // ============================================================================ BFS
 // Level-synchronous top-down BFS (Sec. 4.5 BFS over CSR, through the cache).
-// Level L: app warps claim chunks of 32 to 128 consecutive vertex ids; a lane owns one
-// vertex and takes part when level[v] == L.  Its offsets[v], offsets[v+1] (int64) and
-// its neighbour list (int32) are read through the cache; every neighbour u with
-// level[u] == -1 gets level L+1 by compare-and-swap.  Vertices are visited in id order,
-// so neighbouring lists that share a page are read while the page is resident.
+// Level L: app warps claim chunks of 32 to 128 consecutive vertex ids (up to 1,024 at a level
+// with few vertices); a lane owns one vertex and takes part when level[v] == L.  Its
+// offsets[v], offsets[v+1] (int64) and its neighbour list (int32) are read through the
+// cache; every neighbour u with level[u] == -1 gets level L+1 by compare-and-swap.
+// Vertices are visited in id order, so neighbouring lists that share a page are read while
+// the page is resident.
 // A list of at least kHub entries is not scanned by the warp that found it: it goes
 // to a queue of long lists, cut into slices of kSlice entries that any warp may take,
 // so one hub cannot hold up a level.  Every warp drains that queue before it reaches
@@ -855,7 +855,7 @@ struct BfsAppT {
       uint32_t tot = __reduce_add_sync(kFull, found);
       if (l == 0 && tot) atomicAdd(&d.run->acc[1 + L % 3], (unsigned long long)tot);
       if (l == 0) app_event(d, a.warp, kEvHubsDone, (uint32_t)L);
-      if (!app_barrier(d, a.n_warps, a.deadline)) return;
+      if (!app_barrier(d, a.deadline)) return;
       if (l == 0) app_event(d, a.warp, kEvLevelDone, (uint32_t)L);
       if (aborted(d)) return;
       uint64_t disc = ld_acq64(&d.run->acc[1 + L % 3]);
@@ -863,7 +863,7 @@ struct BfsAppT {
       frontier = disc;
     }
     if (l == 0 && scanned) atomicAdd(&d.run->acc[0], scanned);
-    if (!app_barrier(d, a.n_warps, a.deadline)) return;
+    if (!app_barrier(d, a.deadline)) return;
     if (a.warp == 0 && l == 0 && edges_out) *edges_out = ld_acq64(&d.run->acc[0]);
   }
 };
@@ -1351,7 +1351,7 @@ struct SpmvAppT {
     release(d, pcol);
     release(d, pval);
     if (l == 0 && entries) atomicAdd(&d.run->acc[0], entries);
-    if (!app_barrier(d, a.n_warps, a.deadline)) return;
+    if (!app_barrier(d, a.deadline)) return;
     if (a.warp == 0 && l == 0 && entries_out) *entries_out = ld_acq64(&d.run->acc[0]);
   }
 };
@@ -1373,7 +1373,7 @@ using SpmvApp = SpmvAppT<false>;
 // number of listed bags (the last CTA to finish, which clears the counters for the next
 // call): a small call is two launches, and when everything is resident the second ends at
 // once.  64 bags of 8 resident rows: 18.5 us with a memset, a reset launch and a full
-// engine launch around it, 8 us now.
+// engine launch around it, 10.2 us so.
 template <int MF4>
 __global__ void __launch_bounds__(256, MF4 >= 8 ? 2 : 4) resident_bag_kernel(Dev d, uint64_t page0, uint32_t rows, uint32_t dim,
                                                            const int64_t *idx, const int64_t *off, uint32_t n_bags,

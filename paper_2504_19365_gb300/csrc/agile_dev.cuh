@@ -525,8 +525,7 @@ static __device__ __forceinline__ void sq_ring(const Dev &d, uint32_t q, uint32_
 // slower with it, 3 %).  For one device only (consecutive slots of a queue).
 // False for a lane of a group that found no room.
 static __device__ __forceinline__ bool sq_reserve_group(const Dev &d, bool want, uint32_t q0, uint32_t &q,
-                                                        uint32_t &slot, uint32_t &ticket, uint32_t &first, uint32_t &n,
-                                                        bool pf = false, uint64_t w0 = kNoWord) {
+                                                        uint32_t &slot, uint32_t &ticket, uint32_t &first, uint32_t &n) {
   const unsigned l = lane_id(), base = l & ~3u;
   const uint32_t mine = (__ballot_sync(kFull, want) >> base) & 15u;
   const int lead = (int)base + (mine ? __ffs(mine) - 1 : 0);
@@ -534,7 +533,7 @@ static __device__ __forceinline__ bool sq_reserve_group(const Dev &d, bool want,
   n = 0;
   if (want && lead == (int)l) {
     n = __popc(mine);
-    ok = sq_reserve_dev(d, q0, 0, n, q, slot, ticket, pf, w0);
+    ok = sq_reserve_dev(d, q0, 0, n, q, slot, ticket);
   }
   __syncwarp();
   ok = __shfl_sync(kFull, ok, lead);
@@ -554,7 +553,6 @@ static __device__ __forceinline__ bool sq_reserve_group(const Dev &d, bool want,
 // threads can insert it into different slots.  page * sh_mul mod 2^sh_bits (an odd
 // multiplier: a bijection of the store's page numbers) gives the bucket in its upper bits
 // and the key in its lower 15, so equal keys in a bucket are equal pages.
-constexpr uint64_t SH_FILL = 1, SH_WRITE = 2;
 constexpr uint32_t kShKeyBits = 15;
 __device__ __forceinline__ uint32_t sh_hash(const Dev &d, uint64_t page, uint64_t &key) {
   uint64_t y = (page * d.sh_mul) & ((1ull << d.sh_bits) - 1);
@@ -571,8 +569,7 @@ __device__ __forceinline__ int sh_find(uint64_t word, uint64_t key) {
 // returns slot index >= 0 when inserted, -1 when the page is already present, -2 when
 // the bucket is full (or too contended).  The insertion acquires: what the page's last
 // request wrote before it left the table (tag, store) is seen after it.
-__device__ __forceinline__ int64_t sh_insert(const Dev &d, uint64_t page, uint64_t kind) {
-  (void)kind;
+__device__ __forceinline__ int64_t sh_insert(const Dev &d, uint64_t page) {
   uint64_t key;
   const uint32_t b = sh_hash(d, page, key);
   uint64_t w = 0;  // most buckets are empty
@@ -822,7 +819,7 @@ static __device__ __forceinline__ int pick_victim8(const Dev &d, uint32_t set, c
       }
     if (!zero && (passed >> p & 1u)) tl &= ~(uint32_t)TAG_REF;
     const uint64_t tw = (uint64_t)th << 32 | tl;
-    if ((tl & 3) == ST_MODIFIED) sh_wb = sh_insert(d, tag_page(tw), SH_WRITE);
+    if ((tl & 3) == ST_MODIFIED) sh_wb = sh_insert(d, tag_page(tw));
     if (((tl & 3) != ST_MODIFIED || sh_wb >= 0) &&
         atomicCAS(&tags[w], (unsigned long long)tw, (unsigned long long)claimed) == tw) {
       if (!zero) atomicAdd(&d.hand[set], (first ? 0u : 8u) + p + 1);
@@ -863,7 +860,7 @@ static __device__ __noinline__ int64_t pick_victim(uint32_t set, uint64_t claime
       continue;
     }
     if (st == ST_MODIFIED) {
-      sh_wb = sh_insert(d, tag_page(t), SH_WRITE);
+      sh_wb = sh_insert(d, tag_page(t));
       if (sh_wb < 0) continue;
     }
     if (atomicCAS(&d.tag[base + w], (unsigned long long)t, (unsigned long long)claimed) == t) {
@@ -900,7 +897,7 @@ static __device__ __forceinline__ int cache_claim(const Dev &d, uint64_t page, u
   c.w0 = kNoWord;
   if (fill) {
     c.w0 = sq_first_word(d, q0, dev_of_page(d, page), pf);
-    c.sh = sh_insert(d, page, SH_FILL);
+    c.sh = sh_insert(d, page);
     if (c.sh < 0) {
       // another thread is at the page (a request made without waiting is done with it) or
       // the bucket is full
@@ -1445,7 +1442,7 @@ __device__ __forceinline__ void sum_rows(const Dev &d, uint32_t j0, uint32_t k, 
   }
 }
 
-// Sum-pool rows begin..cnt-1 into acc, added in increasing lane order (lane j holds row
+// Sum-pool rows 0..cnt-1 into acc, added in increasing lane order (lane j holds row
 // j's page `pg` and byte offset `off`).  Lane l adds the float4 columns l, l+32, ... (MF4
 // of them, dim/4 in total).
 // Each round probes the distinct pages of the rows not yet added, without pinning.  Of
@@ -1458,12 +1455,12 @@ __device__ __forceinline__ void sum_rows(const Dev &d, uint32_t j0, uint32_t k, 
 // and adds its row: every round adds at least one row, whatever the set conflicts.
 // `missed` (optional) is set in every lane when some page had to be requested.
 template <int MF4>
-static __device__ bool gather_sum(const Dev &d, const AppCtx &a, uint32_t begin, uint32_t cnt, uint64_t pg, uint32_t off,
-                           uint32_t nf4, float4 (&acc)[MF4], uint32_t window, bool *missed = nullptr) {
+static __device__ bool gather_sum(const Dev &d, const AppCtx &a, uint32_t cnt, uint64_t pg, uint32_t off, uint32_t nf4,
+                                  float4 (&acc)[MF4], uint32_t window, bool *missed = nullptr) {
   unsigned l = lane_id();
-  uint32_t j0 = begin;
+  uint32_t j0 = 0;
   bool first = true;
-  const unsigned grp = __match_any_sync(kFull, l >= begin && l < cnt ? pg : ~0ull);
+  const unsigned grp = __match_any_sync(kFull, l < cnt ? pg : ~0ull);
   while (j0 < cnt) {
     bool act = l >= j0 && l < cnt;
     int lead_lane = __ffs(grp & (~0u << j0)) - 1;  // lowest lane of the page not yet added
@@ -2017,8 +2014,7 @@ static __device__ void poller_loop(const Dev &d, uint32_t q0, uint32_t step, uin
 // Grid barrier over the application warps only (service warps never join).  The warps of a
 // CTA meet in shared memory; the last one of each meets the others' in device memory (a
 // single counter for all 2,000 warps took 5 us of serialised atomics).
-static __device__ bool app_barrier(const Dev &d, uint32_t n_app, uint64_t deadline) {
-  (void)n_app;
+static __device__ bool app_barrier(const Dev &d, uint64_t deadline) {
   CtaState &cs = cta_state();
   bool ok = true;
   __syncwarp();

@@ -29,8 +29,8 @@ __device__ __forceinline__ bool page_ok(const Dev &d, uint64_t page) {
 // before it copies the kPart in front of them, so that the device works while the warp
 // copies.  Many warps with few pages in flight each, because a warp copies in order and a deep
 // queue makes it wait for its next page: 65,536 random pages of which 60 k miss take
-// 1.31 ms with parts of 2, 1.42 of 4, 1.44 of 8 and 1.57 of 16 (bound: the host link,
-// 1.16 ms); 8,192 pages through 4,096 lines 0.27, 0.28, 0.40 and 0.54 ms.
+// 1.31 ms with parts of 2, 1.42 of 4, 1.44 of 8 and 1.57 of 16 (bound: the host link, 1.30 ms
+// at the 189 GB/s that random pages reach); 8,192 pages through 4,096 lines 0.27, 0.28, 0.40 and 0.54 ms.
 struct ReadApp {
   const uint64_t *pages;
   uint32_t n;
@@ -185,7 +185,7 @@ struct WriteApp {
       int64_t sh = -1;
       uint32_t ns = 64;
       for (;;) {
-        if (l == 0) sh = sh_insert(d, page, SH_WRITE);
+        if (l == 0) sh = sh_insert(d, page);
         sh = __shfl_sync(kFull, sh, 0);
         if (sh >= 0) break;
         if (gtimer() > a.deadline || aborted(d)) {
@@ -286,8 +286,8 @@ struct WriteApp {
 // warp repeats its pass until its lines are clean.  Each write-back owns the page's
 // share-table entry until completion.  The device reads the page from the line itself:
 // the write-back bit keeps the line from eviction, and nothing else in this launch writes
-// lines.  8 k dirty lines: 187 us of the 160 that the link needs; copied to staging pages
-// first, by 256 warps of the 2,048, it was 385.
+// lines.  8 k dirty lines: 187 us, of which the link needs 177 (at 189 GB/s); copied to
+// staging pages first, by 256 warps of the 2,048, it was 385.
 struct FlushApp {
   __device__ void run(const Dev &d, const AppCtx &a) const {
     unsigned l = lane_id();
@@ -302,7 +302,7 @@ struct FlushApp {
           t = ld_rlx64(&d.tag[line]);
           if (tag_state(t) == ST_MODIFIED) {
             dirty_left = true;
-            if ((t & (PIN_MASK | TAG_WB)) == 0) sh = sh_insert(d, tag_page(t), SH_WRITE);
+            if ((t & (PIN_MASK | TAG_WB)) == 0) sh = sh_insert(d, tag_page(t));
             // MODIFIED -> READY with the write-back bit: the line stays valid for
             // readers and cannot be evicted until the write completes
             if (sh >= 0 && atomicCAS(&d.tag[line], (unsigned long long)t, (unsigned long long)((t & ~1ull) | TAG_WB)) != t) {
@@ -653,9 +653,7 @@ int agile_init(const agile_config *cfg_in, agile_ctx **out) {
   d.fault_thresh = (uint32_t)fmin(4294967295.0, cfg.fault_rate * 4294967296.0);
   d.seed = cfg.seed;
   d.timeout_ns = cfg.wait_timeout_ns;
-  d.extra_engines = cfg.emu_extra_engines == AGILE_NO_EXTRA_ENGINES
-                        ? 0u
-                        : cfg.emu_extra_engines;
+  d.extra_engines = cfg.emu_extra_engines == AGILE_NO_EXTRA_ENGINES ? 0u : cfg.emu_extra_engines;
   d.prefetch_depth = cfg.prefetch_depth;
   if (cudaDeviceSynchronize() != cudaSuccess) {
     agile_destroy(c);

@@ -160,7 +160,7 @@ struct ServeApp {
       uint64_t byte = r * dim * 4;
       if (mode == AGILE_ASYNC && !warp_request(d, l < cnt, page0 + byte / kPage, a.q0, false, a.deadline))
         return false;
-      if (!gather_sum<1>(d, a, 0, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, window)) return false;
+      if (!gather_sum<1>(d, a, cnt, page0 + byte / kPage, (uint32_t)(byte % kPage), nf4, acc, window)) return false;
     }
     if (l < nf4) ((float4 *)(out + (uint64_t)b * dim))[l] = acc[0];
     return true;

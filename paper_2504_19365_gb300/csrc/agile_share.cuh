@@ -106,7 +106,7 @@ static __device__ __forceinline__ void ub_ready(const Dev &d, uint64_t k, uint64
 // One attempt to fill the new entry k of `page` into `mine`: 1 done (*tok set; a read may
 // have been issued), 0 try again later.
 static __device__ int ub_fill(const Dev &d, const AppCtx &a, uint64_t page, uint8_t *mine, uint64_t k, uint64_t &tok) {
-  int64_t sh = sh_insert(d, page, SH_FILL);
+  int64_t sh = sh_insert(d, page);
   if (sh < 0) return 0;  // the page is in flight (a fill or a write-back): later
   uint32_t line = 0;
   int pr = cache_probe(d, page, true, line);
@@ -141,7 +141,7 @@ static __device__ int ub_fill(const Dev &d, const AppCtx &a, uint64_t page, uint
 // attempts (-1: not taken yet); a write-back of the line's victim may be issued.
 static __device__ int ub_propagate(const Dev &d, const AppCtx &a, uint64_t page, const uint8_t *buf, int64_t &sh) {
   if (sh < 0) {
-    sh = sh_insert(d, page, SH_WRITE);
+    sh = sh_insert(d, page);
     if (sh < 0) return 0;
   }
   uint32_t line = 0;

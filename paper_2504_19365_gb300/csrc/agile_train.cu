@@ -474,7 +474,7 @@ int agile_embedding_bag_backward(agile_ctx *c, uint64_t table_byte0, uint32_t ro
   const uint32_t span = long_span(dim);
   const uint64_t windows = (n + span - 1) / span;
   // scratch: keys before and after a pass, sums of the rows of many positions (16-byte
-  // aligned: n is rounded up to even), counts, totals, bag of each position
+  // aligned: n is rounded up to a multiple of 4), counts, totals, bag of each position
   const uint64_t n2 = (n + 3) & ~3ull;
   const uint64_t g_floats = lr != 0.0f ? windows * dim : 0;
   size_t need = n2 * 16 + g_floats * 4 + (size_t)digits * tiles * 4 + 1024 + n2 * 4;
