@@ -1789,9 +1789,9 @@ int agile_embedding_pipeline(agile_ctx *c, uint64_t table_byte0, uint64_t table_
     // A lookahead adds requests in flight only while the queues have room for more than
     // the warps' own demand.  The running warps' groups of rows are at most run * group
     // reads in flight, about half of that while the warps also compute; when that half
-    // alone fills the queue slots, the call runs as SYNC (measured at the full grid of
-    // 2,128 warps: async 0.93-1.01x sync with the lookahead, its hints mostly dropped
-    // for crowded queues).
+    // alone fills the queue slots, the call runs as SYNC (measured with 2,128 warps in an
+    // earlier launch shape: async 0.93-1.01x sync with the lookahead, its hints mostly
+    // dropped for crowded queues).
     const bool look =
         mode == AGILE_ASYNC && (uint64_t)run * group < 2ull * c->dev.Q * (c->dev.depth - 1);
     uint64_t ahead = look ? c->dev.nlines / (2ull * run) * c->cfg.prefetch_depth : 0;

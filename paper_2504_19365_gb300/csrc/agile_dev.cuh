@@ -1452,8 +1452,8 @@ __device__ __forceinline__ void sum_rows(const Dev &d, uint32_t j0, uint32_t k, 
 // Each round probes the distinct pages of the rows not yet added, without pinning.  Of
 // those not READY, the first `window` ones that nobody has requested are requested
 // without waiting (the window keeps what all running warps have requested and not yet
-// used within the cache; rows that hit do not count, so that a bag of mostly resident
-// rows is one or two rounds).  Then the pages of the leading run of READY rows are
+// used within the cache and the queues; rows that hit do not count, so that a bag of
+// mostly resident rows is one or two rounds).  Then the pages of the leading run of READY rows are
 // pinned, the run is added and every pin let go.  When the next row's page is not READY
 // the warp waits for and pins that one page (nothing else pinned meanwhile, Sec. 2.3.2)
 // and adds its row: every round adds at least one row, whatever the set conflicts.
